@@ -11,8 +11,8 @@
 //    the bucket (the sync-free form: no host read between its launches);
 //  * H_i = sym(W_i^* A_i) and B = H_2 - H_1 per instance (the padded part of
 //    B is exactly zero), and every B of every bucket is one leaf of the
-//    batched one-sided Jacobi eigensolver at its own size, with a fixed
-//    number of sweeps and device-side convergence flags;
+//    batched leaf eigensolver (leaf.cu) at its own size, with a fixed number
+//    of launches and device-side convergence flags;
 //  * C, S = diag(V^* H_i V), theta = atan2(S, C), U_i = W_i V by batched
 //    products on the padded V, then one CTA per instance sorts its angles
 //    and writes its columns into the packed outputs.
@@ -37,7 +37,7 @@ namespace zcsd {
 namespace {
 
 constexpr int BATCH_MAX_N = 1024;
-constexpr int BATCH_SWEEPS = 30;  // Jacobi sweeps of the leaves (converged leaves are skipped)
+constexpr int BATCH_SWEEPS = 30;  // FP64 Jacobi sweeps at most of a leaf that the refinement leaves open
 
 struct Bucket {
   int nb = 0;                    // padded size
@@ -143,7 +143,6 @@ void run_bucket(Ctx& cx, Arena& ar, Bucket& bk, const double* A1, const double* 
   double* H = ar.get<double>(2 * P * nn);
   double* Bm = ar.get<double>(P * nn);
   double* lam = ar.get<double>((size_t)P * nb);
-  double* G = ar.get<double>((size_t)bk.leaves.vtot);
   double* Vl = ar.get<double>((size_t)bk.leaves.vtot);
   double* Vp = ar.get<double>(P * nn);
   double* T1 = ar.get<double>(P * nn);
@@ -171,7 +170,7 @@ void run_bucket(Ctx& cx, Arena& ar, Bucket& bk, const double* A1, const double* 
   axpby<double>(st, nb, nb, 1.0, H + nn, nb, 2 * nn, 0.0, Bm, nb, nn, P);
   axpby<double>(st, nb, nb, -1.0, H, nb, 2 * nn, 1.0, Bm, nb, nn, P);
   // line 5: every B as one leaf of the batched Jacobi eigensolver
-  leaf_solve<double>(cx, bk.leaves, Bm, lam, G, Vl, BATCH_SWEEPS);
+  leaf_solve<double>(cx, ar, bk.leaves, Bm, lam, Vl, BATCH_SWEEPS, true);
   pad_vectors_kernel<<<dim3(gx, P), 256, 0, st>>>(nb, bk.dn, bk.leaves.goff, Vl, Vp);
   ZCSD_LAUNCH();
   // lines 6-9: C, S = diag(V^* H_i V), U_i = W_i V
@@ -233,7 +232,7 @@ namespace {
 size_t bucket_bytes(const Bucket& bk) {
   const long long P = (long long)bk.inst.size(), nb = bk.nb, nn = nb * nb;
   const size_t es = sizeof(double);
-  size_t b = (size_t)(2 * P * nn * 3 + P * nn * 4 + P * nb * 4) * es + (size_t)bk.leaves.vtot * 2 * es;
+  size_t b = (size_t)(2 * P * nn * 3 + P * nn * 4 + P * nb * 4) * es + (size_t)bk.leaves.vtot * 4 * es;
   // zolo_pd on 2P problems plus the tensor-core slices of its largest product
   const long long r = R_MAX;
   const long long qr = 2 * (2 * nn) * 2 * P * r + (long long)ceil_div(nb, NB_OUT) * (nb + 1 + NB_OUT) * NB_OUT * 2 * P * r +
@@ -271,13 +270,13 @@ int build_buckets(csd_batch* b, int gran) {
     b->buckets.push_back(bk);
   }
   // persistent region: per bucket n, off, toff and the leaf tables (index
-  // arrays, shifts, one rotation record of 40 bytes per leaf row); statuses;
-  // instance lists; every allocation rounded up to 256 bytes
+  // arrays, FP32 columns, rotation records); statuses; instance lists; every
+  // allocation rounded up to 256 bytes
   size_t pbytes = 0;
   for (auto& bk : b->buckets) {
-    size_t rows = 0;
-    for (int i : bk.inst) rows += (size_t)b->n[i];
-    pbytes += bk.inst.size() * 128 + rows * 48 + 16 * 256;
+    std::vector<int> sz;
+    for (int i : bk.inst) sz.push_back(b->n[i]);
+    pbytes += bk.inst.size() * 128 + leaf_table_bytes(sz, false) + 16 * 256;
   }
   pbytes += (size_t)b->count * 16 + 4 * 256 + (1 << 20);
   size_t run = 0;
@@ -325,7 +324,7 @@ int build_buckets(csd_batch* b, int gran) {
       ZCSD_CUDA(cudaMemcpyAsync(bk.dn, hn.data(), sizeof(int) * P, cudaMemcpyHostToDevice, cx.stream));
       ZCSD_CUDA(cudaMemcpyAsync(bk.doff, ho.data(), sizeof(long long) * P, cudaMemcpyHostToDevice, cx.stream));
       ZCSD_CUDA(cudaMemcpyAsync(bk.dtoff, ht.data(), sizeof(long long) * P, cudaMemcpyHostToDevice, cx.stream));
-      bk.leaves = leaf_table_build(cx, per, boff, lds, loff, hn);
+      bk.leaves = leaf_table_build(cx, per, boff, lds, loff, hn, false);
     }
     ZCSD_CUDA(cudaMemcpyAsync(b->dinst, all.data(), sizeof(int) * b->count, cudaMemcpyHostToDevice, cx.stream));
     ZCSD_CUDA(cudaStreamSynchronize(cx.stream));

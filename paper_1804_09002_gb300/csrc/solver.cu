@@ -697,7 +697,7 @@ size_t heig_bytes(long long n, size_t es) {
   const long long nn = n * n;
   long long qr = (long long)ceil_div(n, NB_OUT) * (n + NB_OUT) * NB_OUT +
                  (long long)ceil_div(n, NB_OUT) * NB_OUT * NB_OUT + (long long)(5 * NB_OUT + (MAX_SUM + 1) * NB_QR) * n;
-  long long leaves = 2 * (long long)LEAF_MAX * n + 8 * n;  // packed G_l and V_l: sum sz_l^2 <= n * leaf
+  long long leaves = 5 * std::min<long long>(LEAF_MAX, n) * n + 64 * n;  // packed V, T, S, P and FP32 columns: sum sz^2 <= n leaf
   return (size_t)((7 * nn + std::max(qr, leaves)) * es) + polar_bytes(n, 1, es) + (size_t)(3 * n + 2048) * 8 + 64 * 256;
 }
 

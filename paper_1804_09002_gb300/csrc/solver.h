@@ -107,37 +107,53 @@ void canonical_signs(cudaStream_t st, int m1, int m2, int n, int ncols, T* V, in
 template <class T>
 void svd_polar(Ctx& cx, Arena& ar, int n, const T* A, int lda, T* W, int ldw);
 
-// Leaf tables of the batched one-sided Jacobi eigensolver (device arrays in
-// the arena): leaf l is the sz x sz Hermitian block at element offset boff
-// of the B buffer (leading dimension ldb); its eigenvalues go to lam[loff ..]
-// and its G_l, V_l (leading dimension sz) sit at goff in packed buffers of
-// vtot elements.
-struct LeafTable {
+// Leaf tables of the batched eigensolver (leaf.cu; device arrays in the
+// arena): leaf l is the sz x sz Hermitian block at element offset boff of the
+// B buffer (leading dimension ldb); its eigenvalues go to lam[loff ..], its
+// eigenvectors (leading dimension sz) and FP64 work matrices sit at goff in
+// packed buffers of vtot elements, its FP32 columns at woff of w32.
+constexpr int JAC_SWEEPS_MAX = 40;  // sweeps of the FP64 stage at most
+struct LeafDev {
   const long long* boff = nullptr;
   const int* ldb = nullptr;
   const int* loff = nullptr;
   const int* sz = nullptr;
-  const int* pre = nullptr;  // column pairs before leaf l (pre[nl] = total)
   const long long* goff = nullptr;
-  const long long* roff = nullptr;  // per-row rotation records of leaf l at roff[l]
-  char* rows = nullptr;             // rotation records (rtot of them)
-  double* c = nullptr;       // ||B_l||_F (rotation threshold u ||B_l||_F)
-  int* rot = nullptr;        // rotations of leaf l in the current sweep
-  int* done = nullptr;       // leaf l converged
-  int nl = 0, maxsz = 0, maxpad = 0, total_pairs = 0;
-  long long vtot = 0, rtot = 0;
-  double sweep_flops = 0.0;  // three dot products and two column-pair rotations per pair, all leaves
+  const long long* woff = nullptr;
+  const long long* roff = nullptr;  // rotation records of leaf l at roff[l]
+  double* c = nullptr;              // ||B_l||_F
+  int* done = nullptr;              // leaf l converged
+  int* rot = nullptr;               // [l][JAC_SWEEPS_MAX] rotations of a sweep of the FP64 stage
+  int* cosmax = nullptr;            // [l][pass][sweep] largest cosine of an FP32 sweep (float bits)
+  unsigned* off = nullptr;          // [l][look] 0: refinement ended at or before this look
+  const long long* voff = nullptr;  // per-row values of leaf l at voff[l]:
+  double *lam = nullptr, *rho = nullptr, *mean = nullptr, *scale = nullptr;
+  int* label = nullptr;
+  float *w32 = nullptr, *x32 = nullptr;
+  double *part = nullptr, *norms = nullptr;  // norms[2 l]: tr(B_l) / n, [2 l + 1]: about ||B_l||_2
+  char* recs = nullptr;
+  int nl = 0, maxsz = 0;
+  int nv = 1;                  // float4 per lane and column of the FP32 stage
+  int maxblk = 0, maxcols = 0;  // column blocks of a leaf, columns of a block pair (maxima)
+  long long vtot = 0;
+};
+struct LeafTable : LeafDev {
+  std::vector<int> hsz, hldb;  // host copies
+  std::vector<long long> hboff, hgoff;
 };
 LeafTable leaf_table_build(Ctx& cx, Arena& ar, const std::vector<long long>& boff, const std::vector<int>& ldb,
-                           const std::vector<int>& loff, const std::vector<int>& sz);
-// fixed_sweeps > 0: that many sweeps with no device-to-host read (leaves
-// that stop rotating are skipped), for graph capture; 0: until converged.
+                           const std::vector<int>& loff, const std::vector<int>& sz, bool cplx);
+// bytes leaf_table_build takes from its arena, at most
+size_t leaf_table_bytes(const std::vector<int>& sz, bool cplx);
+// Eigenvalues to lam, eigenvectors to V (packed at goff).  sync_free: no
+// device-to-host read, for graph capture.
 template <class T>
-void leaf_solve(Ctx& cx, const LeafTable& L, const T* B, double* lam, T* G, T* V, int fixed_sweeps);
+void leaf_solve(Ctx& cx, Arena& ar, const LeafTable& L, const T* B, double* lam, T* V, int max_sweeps,
+                bool sync_free);
 
-// Eigendecomposition of the diagonal blocks (off[l], sz[l]) of B by
-// one-sided Jacobi, all leaves batched (svd.cu): eigenvalues to
-// lam[off[l] ..], eigenvectors of leaf l to Vl + voff[l] (ld sz[l]).
+// Eigendecomposition of the diagonal blocks (off[l], sz[l]) of B, all leaves
+// batched (leaf.cu): eigenvalues to lam[off[l] ..], eigenvectors of leaf l to
+// Vl + voff[l] (ld sz[l]).
 template <class T>
 void jacobi_eig_leaves(Ctx& cx, Arena& ar, const std::vector<int>& off, const std::vector<int>& sz, const T* B,
                        int ldb, double* lam, T* Vl, std::vector<long long>& voff);
