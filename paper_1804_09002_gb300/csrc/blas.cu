@@ -16,15 +16,17 @@ namespace zcsd {
 
 namespace {
 
-constexpr int BK = 16, NT = 256;
+constexpr int NT = 256;
 
-// Output tile BM x BN (BM * BN = 4096: 16 outputs per thread as a 4 x 4
-// register tile), k-step BK.  BM = 64 (64 x 64 tiles) is the default; BM = 32
-// (32 x 128 tiles) serves the m <= 32 products of the compact-WY updates.
-template <class T, int OPA, int OPB, int BM>
+// Output tile BM x BN, RM x RN outputs per thread (256 threads), k-step BK.
+// The next k-step's operands are loaded into registers before the current
+// one is consumed (not where a thread's complex 4 x 4 outputs fill them).
+template <class T, int OPA, int OPB, int BM, int BN, int RM, int RN, int BK>
 __global__ void __launch_bounds__(NT, 2) gemm_kernel(GemmArgs<T> g) {
-  constexpr int BN = 4096 / BM;
-  constexpr int TX = BM / 4, TY = BN / 4;  // thread grid over the tile
+  constexpr int TX = BM / RM, TY = BN / RN;  // thread grid over the tile
+  static_assert(TX * TY == NT, "256 threads");
+  constexpr int LA = BM * BK / NT, LB = BN * BK / NT;
+  constexpr bool AHEAD = sizeof(T) == 8 || RM * RN < 16;
   const int z = blockIdx.z;
   const int b = z / g.ksplit, ks = z % g.ksplit;
   const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
@@ -32,7 +34,7 @@ __global__ void __launch_bounds__(NT, 2) gemm_kernel(GemmArgs<T> g) {
   if (g.uplo == 2 && n0 > m0 + BM - 1) return;
   int kb = 0, ke = g.k;
   if (g.ksplit > 1) {
-    const int kc = ((g.k + g.ksplit - 1) / g.ksplit + BK - 1) / BK * BK;
+    const int kc = ((g.k + g.ksplit - 1) / g.ksplit + 15) / 16 * 16;
     kb = ks * kc;
     ke = min(g.k, kb + kc);
   }
@@ -45,77 +47,94 @@ __global__ void __launch_bounds__(NT, 2) gemm_kernel(GemmArgs<T> g) {
   __shared__ T Bs[BK][BN + 1];
   const int tid = threadIdx.x;
   const int tx = tid % TX, ty = tid / TX;
-  T acc[4][4];
+  T acc[RM][RN];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < RM; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = zero<T>();
+    for (int j = 0; j < RN; ++j) acc[i][j] = zero<T>();
 
-  for (int js = 0; js < g.nsum; ++js) {
+  T va[LA], vb[LB];
+  const int k00 = (kb / 16) * 16, steps = ke > k00 ? (ke - k00 + BK - 1) / BK : 0;
+  // ---- op(A)[m0:m0+BM, kt:kt+BK] and op(B)[kt:kt+BK, n0:n0+BN] into
+  // registers, coalesced along memory
+  auto fetch = [&](int it) {
+    const int js = it / steps, kt = k00 + (it % steps) * BK;
     const T* A = g.A + (b / g.bdivA) * g.sA + js * g.sAj;
     const T* B = g.B + (b / g.bdivB) * g.sB + js * g.sBj;
     const double wj = g.w[js];
-    for (int kt = (kb / BK) * BK; kt < ke; kt += BK) {
-      // ---- op(A)[m0:m0+BM, kt:kt+BK] -> As[k][i], coalesced along memory
 #pragma unroll
-      for (int s = 0; s < (BM * BK) / NT; ++s) {
-        const int e = tid + NT * s;
-        const int i = (OPA == OP_N) ? (e % BM) : (e / BK);
-        const int k = (OPA == OP_N) ? (e / BM) : (e % BK);
-        const int gi = m0 + i, gk = kt + k;
-        T v = zero<T>();
-        if (gi < g.m && gk >= kb && gk < ke) {
-          if (OPA == OP_N) v = A[gi + (long long)gk * g.lda];
-          else {
-            v = A[gk + (long long)gi * g.lda];
-            if (OPA == OP_C) v = conj_(v);
-          }
+    for (int s = 0; s < LA; ++s) {
+      const int e = tid + NT * s;
+      const int i = (OPA == OP_N) ? (e % BM) : (e / BK);
+      const int k = (OPA == OP_N) ? (e / BM) : (e % BK);
+      const int gi = m0 + i, gk = kt + k;
+      T v = zero<T>();
+      if (gi < g.m && gk >= kb && gk < ke) {
+        if (OPA == OP_N) v = A[gi + (long long)gk * g.lda];
+        else {
+          v = A[gk + (long long)gi * g.lda];
+          if (OPA == OP_C) v = conj_(v);
         }
-        As[k][i] = scal(wj, v);
       }
-      // ---- op(B)[kt:kt+BK, n0:n0+BN] -> Bs[k][j]
-#pragma unroll
-      for (int s = 0; s < (BN * BK) / NT; ++s) {
-        const int e = tid + NT * s;
-        const int k = (OPB == OP_N) ? (e % BK) : (e / BN);
-        const int j = (OPB == OP_N) ? (e / BK) : (e % BN);
-        const int gj = n0 + j, gk = kt + k;
-        T v = zero<T>();
-        if (gj < g.n && gk >= kb && gk < ke) {
-          if (OPB == OP_N) v = B[gk + (long long)gj * g.ldb];
-          else {
-            v = B[gj + (long long)gk * g.ldb];
-            if (OPB == OP_C) v = conj_(v);
-          }
-        }
-        Bs[k][j] = v;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int k = 0; k < BK; ++k) {
-        T a[4], bb[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = As[k][tx + TX * i];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) bb[j] = Bs[k][ty + TY * j];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = fmac(a[i], bb[j], acc[i][j]);
-      }
-      __syncthreads();
+      va[s] = scal(wj, v);
     }
+#pragma unroll
+    for (int s = 0; s < LB; ++s) {
+      const int e = tid + NT * s;
+      const int k = (OPB == OP_N) ? (e % BK) : (e / BN);
+      const int j = (OPB == OP_N) ? (e / BK) : (e % BN);
+      const int gj = n0 + j, gk = kt + k;
+      T v = zero<T>();
+      if (gj < g.n && gk >= kb && gk < ke) {
+        if (OPB == OP_N) v = B[gk + (long long)gj * g.ldb];
+        else {
+          v = B[gj + (long long)gk * g.ldb];
+          if (OPB == OP_C) v = conj_(v);
+        }
+      }
+      vb[s] = v;
+    }
+  };
+  const int total = steps * g.nsum;
+  if (AHEAD && total > 0) fetch(0);
+  for (int it = 0; it < total; ++it) {
+    if (!AHEAD) fetch(it);
+#pragma unroll
+    for (int s = 0; s < LA; ++s) {
+      const int e = tid + NT * s;
+      As[(OPA == OP_N) ? (e / BM) : (e % BK)][(OPA == OP_N) ? (e % BM) : (e / BK)] = va[s];
+    }
+#pragma unroll
+    for (int s = 0; s < LB; ++s) {
+      const int e = tid + NT * s;
+      Bs[(OPB == OP_N) ? (e % BK) : (e / BN)][(OPB == OP_N) ? (e / BK) : (e % BN)] = vb[s];
+    }
+    __syncthreads();
+    if (AHEAD && it + 1 < total) fetch(it + 1);
+#pragma unroll
+    for (int k = 0; k < BK; ++k) {
+      T a[RM], bb[RN];
+#pragma unroll
+      for (int i = 0; i < RM; ++i) a[i] = As[k][tx + TX * i];
+#pragma unroll
+      for (int j = 0; j < RN; ++j) bb[j] = Bs[k][ty + TY * j];
+#pragma unroll
+      for (int i = 0; i < RM; ++i)
+#pragma unroll
+        for (int j = 0; j < RN; ++j) acc[i][j] = fmac(a[i], bb[j], acc[i][j]);
+    }
+    __syncthreads();
   }
   // ---- epilogue
   T* C = g.C + z * g.sC;
   const T* Cin = g.Cin ? g.Cin + (b / g.bdivC) * g.sCin : nullptr;
   const bool use_beta = Cin && ks == 0 && (re(g.beta) != 0.0 || im(g.beta) != 0.0);
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < RN; ++j) {
     const int gj = n0 + ty + TY * j;
     if (gj >= g.n) continue;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < RM; ++i) {
       const int gi = m0 + tx + TX * i;
       if (gi >= g.m) continue;
       T v = mul(g.alpha, acc[i][j]);
@@ -125,24 +144,58 @@ __global__ void __launch_bounds__(NT, 2) gemm_kernel(GemmArgs<T> g) {
   }
 }
 
-template <class T, int OPA, int BM>
-void gemm_dispatch_b(const GemmArgs<T>& g, cudaStream_t st) {
-  constexpr int BN = 4096 / BM;
-  dim3 grid(ceil_div(g.m, BM), ceil_div(g.n, BN), g.batch * g.ksplit);
-  switch (g.opB) {
-    case OP_N: gemm_kernel<T, OPA, OP_N, BM><<<grid, NT, 0, st>>>(g); break;
-    case OP_T: gemm_kernel<T, OPA, OP_T, BM><<<grid, NT, 0, st>>>(g); break;
-    default: gemm_kernel<T, OPA, OP_C, BM><<<grid, NT, 0, st>>>(g); break;
+// Tiles of the FP64 product.  The pipe (two multiply-adds per clock and SM) is
+// the bound at every tile size, one output per thread included, so the tile
+// is the one whose fullest SM has the least to do: ceil(tiles / 152) tiles of
+// BM x BN outputs.  128^3 (two problems): 64 x 64 tiles on 8 SMs take 130 us,
+// 16 x 16 tiles 9 us.  Large outputs keep 64 x 64 (32 x 128 for m <= 32),
+// which read each operand least often; a smaller tile has to win by 10 %.
+// A product in place needs one tile over the whole of what it overwrites.
+enum GemmTile { TILE_64 = 0, TILE_32x128, TILE_32, TILE_16, TILES };
+constexpr int TILE_M[TILES] = {64, 32, 32, 16}, TILE_N[TILES] = {64, 128, 32, 16};
+
+template <class T>
+int pick_tile(const GemmArgs<T>& g) {
+  int best = -1;
+  double cost = 0.0;
+  for (int t = 0; t < TILES; ++t) {
+    if ((g.C == g.B && TILE_M[t] < g.m) || (g.C == g.A && TILE_N[t] < g.n)) continue;
+    const long long tm = ceil_div(g.m, TILE_M[t]), tn = ceil_div(g.n, TILE_N[t]);
+    long long tiles = tm * tn;
+    if (g.uplo) tiles = (tiles + std::min(tm, tn)) / 2;
+    tiles *= (long long)g.batch * g.ksplit;
+    const double c = (double)ceil_div(tiles, 152) * TILE_M[t] * TILE_N[t];
+    if (best < 0 || c < 0.9 * cost) {
+      best = t;
+      cost = c;
+    }
+  }
+  return best < 0 ? TILE_64 : best;
+}
+
+template <class T, int OPA, int OPB>
+void gemm_launch(const GemmArgs<T>& g, int tile, cudaStream_t st) {
+  const dim3 grid(ceil_div(g.m, TILE_M[tile]), ceil_div(g.n, TILE_N[tile]), g.batch * g.ksplit);
+  switch (tile) {
+    case TILE_64: gemm_kernel<T, OPA, OPB, 64, 64, 4, 4, 16><<<grid, NT, 0, st>>>(g); break;
+    case TILE_32x128: gemm_kernel<T, OPA, OPB, 32, 128, 4, 4, 16><<<grid, NT, 0, st>>>(g); break;
+    case TILE_32: gemm_kernel<T, OPA, OPB, 32, 32, 2, 2, 16><<<grid, NT, 0, st>>>(g); break;
+    default: gemm_kernel<T, OPA, OPB, 16, 16, 1, 1, 32><<<grid, NT, 0, st>>>(g); break;
   }
 }
 
-template <class T, int BM>
-void gemm_dispatch(const GemmArgs<T>& g, cudaStream_t st) {
-  switch (g.opA) {
-    case OP_N: gemm_dispatch_b<T, OP_N, BM>(g, st); break;
-    case OP_T: gemm_dispatch_b<T, OP_T, BM>(g, st); break;
-    default: gemm_dispatch_b<T, OP_C, BM>(g, st); break;
-  }
+template <class T, int OPA>
+void gemm_dispatch_b(const GemmArgs<T>& g, int tile, cudaStream_t st) {
+  if (g.opB == OP_N) gemm_launch<T, OPA, OP_N>(g, tile, st);
+  else if (g.opB == OP_C && sizeof(T) == 16) gemm_launch<T, OPA, OP_C>(g, tile, st);
+  else gemm_launch<T, OPA, OP_T>(g, tile, st);
+}
+
+template <class T>
+void gemm_dispatch(const GemmArgs<T>& g, int tile, cudaStream_t st) {
+  if (g.opA == OP_N) gemm_dispatch_b<T, OP_N>(g, tile, st);
+  else if (g.opA == OP_C && sizeof(T) == 16) gemm_dispatch_b<T, OP_C>(g, tile, st);
+  else gemm_dispatch_b<T, OP_T>(g, tile, st);
 }
 
 // Multiply-add work the kernel executes for g, counted per output tile over
@@ -184,12 +237,11 @@ void gemm(const GemmArgs<T>& g, cudaStream_t st) {
       return;
     }
   }
-  const bool narrow = g.m <= 32;
   ProfToken tok = prof_begin(st);
-  if (narrow) gemm_dispatch<T, 32>(g, st);
-  else gemm_dispatch<T, 64>(g, st);
+  const int tile = pick_tile(g);
+  gemm_dispatch<T>(g, tile, st);
   ZCSD_LAUNCH();
-  if (tok.slot >= 0) prof_end(tok, st, PK_GEMM, narrow ? gemm_flops(g, 32, 128) : gemm_flops(g, 64, 64), g.site);
+  if (tok.slot >= 0) prof_end(tok, st, PK_GEMM, gemm_flops(g, TILE_M[tile], TILE_N[tile]), g.site);
 }
 
 template <class T>
