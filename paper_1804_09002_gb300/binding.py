@@ -57,8 +57,8 @@ class csd_profile(ctypes.Structure):
                 ("site_flops", ctypes.c_double * 24)]
 
     SITES = ["other", "qr_W", "qr_W2", "qr_update", "formq_W", "formq_W2", "formq_update", "zolo_combine",
-             "gram", "chol_row", "chol_trailing", "trsm_f_update", "trsm_f_diag", "trsm_b_update",
-             "trsm_b_diag", "H", "orth", "eig", "assembly", "alg2", "tmerge", "qr_update_x", "grad"]
+             "gram", "chol_inverse", "chol_trailing", "inverse_sum", "zolo_q", "inverse_apply",
+             "zolo_gram2", "H", "orth", "eig", "assembly", "alg2", "tmerge", "zolo_polish", "grad"]
 
 
 def _load():

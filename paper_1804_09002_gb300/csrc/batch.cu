@@ -154,7 +154,7 @@ void run_bucket(Ctx& cx, Arena& ar, Bucket& bk, const double* A1, const double* 
   pad_gather_kernel<<<dim3(gx, 2 * P), 256, 0, st>>>(nb, P, bk.dn, bk.doff, A1, A2, X);
   ZCSD_LAUNCH();
   // lines 1-2 of Algorithm 1 for every block of every instance
-  zolo_pd<double>(cx, ar, nb, 2 * P, X, W, nullptr, 0, 0, true);
+  zolo_pd<double>(cx, ar, nb, 2 * P, X, W, nullptr);
   {
     GemmArgs<double> g;  // H = sym(W^* X)
     g.batch = 2 * P;
@@ -234,13 +234,8 @@ size_t bucket_bytes(const Bucket& bk) {
   const size_t es = sizeof(double);
   size_t b = (size_t)(2 * P * nn * 3 + P * nn * 4 + P * nb * 4) * es + (size_t)bk.leaves.vtot * 4 * es;
   // zolo_pd on 2P problems plus the tensor-core slices of its largest product
-  const long long r = R_MAX;
-  const long long qr = 2 * (2 * nn) * 2 * P * r + (long long)ceil_div(nb, NB_OUT) * (nb + 1 + NB_OUT) * NB_OUT * 2 * P * r +
-                       (long long)ceil_div(nb, NB_OUT) * NB_OUT * NB_OUT * 2 * P * r +
-                       (long long)(5 * NB_OUT + (MAX_SUM + 1) * NB_QR) * nb * 2 * P * r;
-  const long long ch = nn * 2 * P + 3 * nn * 2 * P * r + (long long)NB_CHOL * nb * 2 * P * r * (2 + MAX_SUM);
-  b += (size_t)(2 * nn * 2 * P + std::max(qr, ch)) * es;
-  b += (size_t)(2 * 14) * (nb + 128) * (2 * nb + 64) * 2 * P * r;  // BF16 slices of the stacked products
+  b += (size_t)(nn * 2 * P * (6 * R_MAX + 6)) * es;
+  b += (size_t)(2 * 14) * (nb + 128) * (nb + 64) * 2 * P * R_MAX;
   return b + ((size_t)64 << 20);
 }
 

@@ -322,31 +322,40 @@ void shift_terms(cudaStream_t st, int n, const T* X, int ldx, long long sXb, con
 }
 
 template <class T>
-void stack_terms(cudaStream_t st, int n, const T* X, int ldx, long long sXb, const double* sqrtc, int nterms,
-                 T* M, int ldm, long long sM, int batch) {
-  Vec16 s;
-  for (int j = 0; j < MAX_SUM; ++j) s.v[j] = j < nterms ? sqrtc[j] : 0.0;
-  ew2d(st, 2 * n, n, batch * nterms, [=] __device__(int i, int j, int p) {
-    const int bb = p / nterms, jt = p % nterms;
-    T v;
-    if (i < n) v = X[bb * sXb + i + (long long)j * ldx];
-    else v = (i - n == j) ? from_re<T>(s.v[jt]) : zero<T>();
-    M[p * sM + i + (long long)j * ldm] = v;
+void scale_shift(cudaStream_t st, int n, double alpha, const T* X, int ldx, long long sX, double beta, T* Z, int ldz,
+                 long long sZ, int batch) {
+  ew2d(st, n, n, batch, [=] __device__(int i, int j, int b) {
+    T x = scal(alpha, X[b * sX + i + (long long)j * ldx]);
+    if (i == j) x = add(x, from_re<T>(beta));
+    Z[b * sZ + i + (long long)j * ldz] = x;
   });
 }
 
 template <class T>
-void sum_terms(cudaStream_t st, int n, double mhat, const T* X1, int ldx, long long sXb, const double* a,
-               int nterms, const T* Tm, int ldt, long long sT, T* X2, int ldx2, long long sX2b, int batch) {
+void scale_terms(cudaStream_t st, int m, int n, const double* s_, int nterms, T* X, int ldx, long long sX, int batch) {
   Vec16 s;
-  for (int j = 0; j < MAX_SUM; ++j) s.v[j] = j < nterms ? a[j] : 0.0;
+  for (int j = 0; j < MAX_SUM; ++j) s.v[j] = j < nterms ? s_[j] : 0.0;
+  ew2d(st, m, n, batch * nterms, [=] __device__(int i, int j, int p) {
+    T* x = X + p * sX + i + (long long)j * ldx;
+    *x = scal(s.v[p % nterms], *x);
+  });
+}
+
+template <class T>
+void minus_eye(cudaStream_t st, int n, const T* X, int ldx, long long sX, T* E, int lde, long long sE, int batch) {
   ew2d(st, n, n, batch, [=] __device__(int i, int j, int b) {
-    T acc = X1[b * sXb + i + (long long)j * ldx];
-    for (int t = 0; t < nterms; ++t) {
-      const T v = Tm[(long long)(b * nterms + t) * sT + i + (long long)j * ldt];
-      acc = add(acc, scal(s.v[t], v));
-    }
-    X2[b * sX2b + i + (long long)j * ldx2] = scal(mhat, acc);
+    if (i > j) return;
+    T x = X[b * sX + i + (long long)j * ldx];
+    if (i == j) x = from_re<T>(re(x) - 1.0);
+    E[b * sE + i + (long long)j * lde] = x;
+    if (i < j) E[b * sE + j + (long long)i * lde] = conj_(x);
+  });
+}
+
+template <class T>
+void mirror(cudaStream_t st, int n, T* X, int ldx, long long sX, int batch) {
+  ew2d(st, n, n, batch, [=] __device__(int i, int j, int b) {
+    if (i < j) X[b * sX + j + (long long)i * ldx] = conj_(X[b * sX + i + (long long)j * ldx]);
   });
 }
 
@@ -622,10 +631,10 @@ void randn(cudaStream_t st, int m, int n, T* X, int ldx, unsigned long long seed
   template void sum_parts<T>(cudaStream_t, int, int, T*, int, long long, int, int);                                  \
   template void shift_terms<T>(cudaStream_t, int, const T*, int, long long, const double*, int, T*, int, long long, \
                                int);                                                                            \
-  template void stack_terms<T>(cudaStream_t, int, const T*, int, long long, const double*, int, T*, int, long long, \
-                               int);                                                                            \
-  template void sum_terms<T>(cudaStream_t, int, double, const T*, int, long long, const double*, int, const T*, int, \
-                             long long, T*, int, long long, int);                                               \
+  template void scale_shift<T>(cudaStream_t, int, double, const T*, int, long long, double, T*, int, long long, int); \
+  template void scale_terms<T>(cudaStream_t, int, int, const double*, int, T*, int, long long, int);            \
+  template void minus_eye<T>(cudaStream_t, int, const T*, int, long long, T*, int, long long, int);             \
+  template void mirror<T>(cudaStream_t, int, T*, int, long long, int);                                          \
   template void symmetrize<T>(cudaStream_t, int, const T*, int, long long, T*, int, long long, int);            \
   template void set_eye<T>(cudaStream_t, int, int, T*, int, long long, int);                                    \
   template void fro2<T>(cudaStream_t, int, int, const T*, int, long long, double, double*, int, double*);       \

@@ -501,62 +501,80 @@ void launch_panel_smem(cudaStream_t st, int m, int n, int band, T* M, int ldm, l
                                chunk));
 }
 
-constexpr int CHOL_MAXNB = 64;
-
+// N = L^{-*} of the lower Cholesky factor of an nb x nb block (nb <= 64), one
+// CTA per problem.  Unscaled elimination of [Z | I]: at pivot j every row
+// i > j loses conj(z_ji) / z_jj times row j; then row i of L^{-1} is row i of
+// the right half over sqrt(z_ii).  Column c of the left half is used up to
+// pivot c and column c of the right half from there on, so both share one
+// nb x nb array held in the registers of 1024 threads.  One barrier per pivot:
+// the threads of the next row publish it and its reciprocal pivot as they
+// finish it.  Bound by the FP64 pipe of one SM (a 64-row block: 87 k
+// multiply-adds, 21 us at two per clock) and the chain of 64 pivots.  A warp's
+// FP64 instruction holds its scheduler for 64 clocks, so the rows are spread
+// over 32 warps (two rows each): 77 us a block, where eight warps of eight
+// rows took 104 us and the factor and its inverse by substitution 310 us.
+// (32-row blocks take 30 us but need four more products per 64 columns: no
+// faster.  Complex blocks have 32 rows: 48 us, 64 rows took 237.)
 template <class T>
-__global__ void __launch_bounds__(256) potrf_inv_kernel(int n, T* Aall, int lda, long long sA, int k0, int nb,
-                                                        T* Rall, int ldr, long long sR, int* info) {
-  extern __shared__ __align__(16) unsigned char dyn_smem[];
-  T(*S)[CHOL_MAXNB + 1] = reinterpret_cast<T(*)[CHOL_MAXNB + 1]>(dyn_smem);
-  T(*X)[CHOL_MAXNB + 1] = S + CHOL_MAXNB;
-  __shared__ int bad;
-  const int b = blockIdx.x;
-  T* A = Aall + b * sA;
-  T* Rinv = Rall + b * sR;
-  const int tid = threadIdx.x;
-  if (tid == 0) bad = 0;
-  for (int t = tid; t < nb * nb; t += blockDim.x) {
-    const int i = t % nb, j = t / nb;
-    S[i][j] = (i <= j) ? A[(k0 + i) + (long long)(k0 + j) * lda] : zero<T>();
-    X[i][j] = zero<T>();
+__global__ void __launch_bounds__(1024) chol_inv_kernel(int nb, const T* Zall, int ldz, long long sZ, T* Nall, int ldn,
+                                                       long long sN) {
+  constexpr int NB = chol_nb<T>(), TPR = 1024 / NB, EN = NB / TPR;  // threads per row, entries per thread
+  constexpr int RPW = 32 / TPR;                                     // rows of a warp
+  __shared__ T row[2][NB];
+  __shared__ double inv[2];
+  const T* Zb = Zall + blockIdx.x * sZ;
+  T* N = Nall + blockIdx.x * sN;
+  const int tid = threadIdx.x, i = tid / TPR, sub = tid % TPR, iw = i / RPW * RPW;
+  T m[EN];
+#pragma unroll
+  for (int k = 0; k < EN; ++k) {
+    const int c = sub + TPR * k;
+    m[k] = (i < nb && c < nb && i <= c) ? Zb[i + (long long)c * ldz] : zero<T>();
   }
-  __syncthreads();
-  // upper Cholesky, row by row: R[j, j:] from S[j, j:] - sum_{p<j} conj(R[p, j]) R[p, j:]
-  for (int j = 0; j < nb; ++j) {
-    if (tid == 0) {
-      double dd = re(S[j][j]);
-      for (int p = 0; p < j; ++p) dd -= abs2(S[p][j]);
-      if (!(dd > 0.0) || !isfinite(dd)) {
-        if (!bad) bad = k0 + j + 1;
-        dd = 1.0;
+  // 1 / x to rounding: FP32 seed, two Newton steps (NaN unless x > 0)
+  auto recip = [](double x) {
+    if (!(x > 0.0)) return (double)NAN;
+    if (!(x > 1e-30 && x < 1e30)) return 1.0 / x;
+    double r = (double)__frcp_rn((float)x);
+    r = fma(r, fma(-x, r, 1.0), r);
+    return fma(r, fma(-x, r, 1.0), r);
+  };
+  auto publish = [&](int j) {  // by the threads of row j
+#pragma unroll
+    for (int k = 0; k < EN; ++k) {
+      const int c = sub + TPR * k;
+      row[j & 1][c] = m[k];
+      if (c == j) inv[j & 1] = recip(re(m[k]));
+    }
+  };
+  if (i == 0) publish(0);
+  for (int j = 0; j + 1 < nb; ++j) {
+    __syncthreads();
+    if (i > j && i < nb) {
+      const T f = scal(-inv[j & 1], conj_(row[j & 1][i]));
+#pragma unroll
+      for (int k = 0; k < EN; ++k) {
+        if (TPR * k > j && TPR * k + TPR - 1 < iw) continue;  // below the diagonal of the left half
+        const int c = sub + TPR * k;
+        m[k] = c == j ? f : fmac(f, row[j & 1][c], m[k]);
       }
-      S[j][j] = from_re<T>(sqrt(dd));
-    }
-    __syncthreads();
-    const double rjj = re(S[j][j]);
-    for (int c = j + 1 + tid; c < nb; c += blockDim.x) {
-      T s = S[j][c];
-      for (int p = 0; p < j; ++p) s = sub(s, cmul(S[p][j], S[p][c]));
-      S[j][c] = scal(1.0 / rjj, s);
-    }
-    __syncthreads();
-  }
-  // R^{-1}: column c by back substitution (one thread per column)
-  for (int c = tid; c < nb; c += blockDim.x) {
-    X[c][c] = from_re<T>(1.0 / re(S[c][c]));
-    for (int i = c - 1; i >= 0; --i) {
-      T s = zero<T>();
-      for (int p = i + 1; p <= c; ++p) s = fmac(S[i][p], X[p][c], s);
-      X[i][c] = scal(-1.0 / re(S[i][i]), s);
+      if (i == j + 1) publish(i);
     }
   }
-  __syncthreads();
-  for (int t = tid; t < nb * nb; t += blockDim.x) {
-    const int i = t % nb, j = t / nb;
-    if (i <= j) A[(k0 + i) + (long long)(k0 + j) * lda] = S[i][j];
-    Rinv[i + (long long)j * ldr] = (i <= j) ? X[i][j] : zero<T>();
+  if (i < nb) {
+    double d = 0.0;
+#pragma unroll
+    for (int k = 0; k < EN; ++k)
+      if (sub + TPR * k == i) d = re(m[k]);
+    d = __shfl_sync(__activemask(), d, (tid & 31) / TPR * TPR + i % TPR);
+    const double s = d > 0.0 ? 1.0 / sqrt(d) : (double)NAN;
+#pragma unroll
+    for (int k = 0; k < EN; ++k) {
+      const int c = sub + TPR * k;
+      if (c < i) N[c + (long long)i * ldn] = scal(s, conj_(m[k]));
+      else if (c == i) N[c + (long long)i * ldn] = from_re<T>(s);
+    }
   }
-  if (tid == 0 && bad && info[b] == 0) info[b] = bad;
 }
 
 }  // namespace
@@ -600,17 +618,11 @@ void qr_panel(cudaStream_t st, int m, int n, int band, T* M, int ldm, long long 
 }
 
 template <class T>
-void potrf_inv(cudaStream_t st, int n, T* A, int lda, long long sA, int k0, int nb, T* Rinv, int ldr,
-               long long sR, int* info, int batch) {
-  if (nb > CHOL_MAXNB) throw CudaFail{cudaErrorInvalidValue, __FILE__, __LINE__};
-  const int smem = 2 * CHOL_MAXNB * (CHOL_MAXNB + 1) * (int)sizeof(T);
-  static const bool attr_set = [smem] {
-    ZCSD_CUDA(cudaFuncSetAttribute(potrf_inv_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    return true;
-  }();
-  (void)attr_set;
+void chol_inv_block(cudaStream_t st, int nb, const T* Z, int ldz, long long sZ, T* N, int ldn, long long sN,
+                    int batch) {
+  if (nb > chol_nb<T>()) throw CudaFail{cudaErrorInvalidValue, __FILE__, __LINE__};
   ProfToken tok = prof_begin(st);
-  potrf_inv_kernel<T><<<batch, 256, smem, st>>>(n, A, lda, sA, k0, nb, Rinv, ldr, sR, info);
+  chol_inv_kernel<T><<<batch, 1024, 0, st>>>(nb, Z, ldz, sZ, N, ldn, sN);
   ZCSD_LAUNCH();
   if (tok.slot >= 0) prof_end(tok, st, PK_POTRF, (2.0 / 3.0) * nb * nb * nb * batch);
 }
@@ -618,7 +630,7 @@ void potrf_inv(cudaStream_t st, int n, T* A, int lda, long long sA, int k0, int 
 #define ZCSD_INST_F(T)                                                                                        \
   template void qr_panel<T>(cudaStream_t, int, int, int, T*, int, long long, int, int, T*, int, long long, T*, \
                             long long, int);                                                                 \
-  template void potrf_inv<T>(cudaStream_t, int, T*, int, long long, int, int, T*, int, long long, int*, int);
+  template void chol_inv_block<T>(cudaStream_t, int, const T*, int, long long, T*, int, long long, int);
 
 ZCSD_INST_F(double)
 ZCSD_INST_F(z64)

@@ -1,5 +1,5 @@
-// Blocked Householder QR (compact WY), blocked Cholesky and the paired
-// triangular solves, as sequences of panel kernels and batched GEMMs.
+// Blocked Householder QR (compact WY) and the recursive inverse Cholesky
+// factor, as sequences of panel kernels and batched GEMMs.
 #include <type_traits>
 
 #include "linalg.h"
@@ -70,7 +70,7 @@ QRStore<T> qr_alloc(Arena& ar, int m, int n, int band, int batch) {
 template <class T>
 static void wy_apply(cudaStream_t st, Arena& ar, int h, int nc, int nb, const T* Y, int ldy, long long sY,
                      const T* Tm, int ldt, long long sT, bool adjoint, T* C, int ldc, long long sC, int batch,
-                     int site_w, int site_w2, int site_upd, int xrows = 0) {
+                     int site_w, int site_w2, int site_upd) {
   if (nc <= 0 || nb <= 0 || h <= 0) return;
   const int kcap = std::min(nb > NB_QR ? 4 : MAX_SUM, std::max(1, h / 256));
   const size_t mk = ar.mark();
@@ -100,24 +100,18 @@ static void wy_apply(cudaStream_t st, Arena& ar, int h, int nc, int nb, const T*
   g2.site = site_w2;
   g2.alpha = one; g2.beta = zer;
   gemm(g2, st);
-  // C -= Y W2; for a stacked [X; sqrt(c) I] the rows of the X block and the
-  // rows below it are separate products (sites GS_QR_UPD_X and site_upd)
-  const int hx = std::min(std::max(xrows, 0), h);
-  for (int part = 0; part < 2; ++part) {
-    const int r0 = part == 0 ? 0 : hx, r1 = part == 0 ? hx : h;
-    if (r1 <= r0) continue;
-    GemmArgs<T> g3;
-    g3.batch = batch;
-    g3.m = r1 - r0; g3.n = nc; g3.k = nb; g3.opA = OP_N; g3.opB = OP_N;
-    g3.A = Y + r0; g3.lda = ldy; g3.sA = sY;
-    g3.B = W2; g3.ldb = nb; g3.sB = sW;
-    g3.Cin = C + r0; g3.ldcin = ldc; g3.sCin = sC;
-    g3.C = C + r0; g3.ldc = ldc; g3.sC = sC;
-    g3.site = part == 0 ? GS_QR_UPD_X : site_upd;
-    g3.kbal = part == 0 ? 0 : 1;  // rows of the size of sqrt(c): balance k on the tensor cores
-    g3.alpha = mone; g3.beta = one;
-    gemm(g3, st);
-  }
+  // C -= Y W2
+  GemmArgs<T> g3;
+  g3.batch = batch;
+  g3.m = h; g3.n = nc; g3.k = nb; g3.opA = OP_N; g3.opB = OP_N;
+  g3.A = Y; g3.lda = ldy; g3.sA = sY;
+  g3.B = W2; g3.ldb = nb; g3.sB = sW;
+  g3.Cin = C; g3.ldcin = ldc; g3.sCin = sC;
+  g3.C = C; g3.ldc = ldc; g3.sC = sC;
+  g3.site = site_upd;
+  g3.kbal = 1;  // rows of any size: balance k on the tensor cores
+  g3.alpha = mone; g3.beta = one;
+  gemm(g3, st);
   ar.release(mk);
 }
 
@@ -159,7 +153,7 @@ void qr_factor(cudaStream_t st, Arena& ar, QRStore<T>& q, T* M, int ldm, long lo
       if (nc_in > 0) {
         const int hi = std::min(m, k0 + nb - 1 + q.band) - k0;
         wy_apply<T>(st, ar, hi, nc_in, nb, Yi, q.ldy, q.sY, Ti, NBO, q.sT, true, M + k0 + (long long)(k0 + nb) * ldm,
-                    ldm, sM, q.batch, GS_QR_W, GS_QR_W2, GS_QR_UPD, q.xrows - k0);
+                    ldm, sM, q.batch, GS_QR_W, GS_QR_W2, GS_QR_UPD);
       }
     }
     // merge the panel factors into the block's T: one Gram matrix
@@ -200,7 +194,7 @@ void qr_factor(cudaStream_t st, Arena& ar, QRStore<T>& q, T* M, int ldm, long lo
     const int nc = n - (K0 + nbo);
     if (nc > 0)
       wy_apply<T>(st, ar, hb, nc, nbo, Yb, q.ldy, q.sY, Tb, NBO, q.sT, true, M + K0 + (long long)(K0 + nbo) * ldm,
-                  ldm, sM, q.batch, GS_QR_W, GS_QR_W2, GS_QR_UPD, q.xrows - K0);
+                  ldm, sM, q.batch, GS_QR_W, GS_QR_W2, GS_QR_UPD);
   }
   ar.release(mk);
 }
@@ -222,169 +216,99 @@ void qr_form_q(cudaStream_t st, Arena& ar, const QRStore<T>& q, T* E, int lde, l
   }
 }
 
-// Rows [r0, r1) of R times columns [j0, j1): Z[r0:r1, j0:j1] <- R11^{-*}
-// Z[r0:r1, j0:j1] with R11 = R[r0:r1, r0:r1] (its lower-triangular adjoint
-// solved recursively: X1 = Ra^{-*} Z1, Z2 -= Rb^* X1, X2 = Rc^{-*} Z2); leaves
-// multiply in place by the inverted diagonal block (one row tile covers it).
+// Columns [c0, c1) of N = R^{-1}, R^* R = Z: invert the leading half, W =
+// N11^* Z12 (= R12), Z22 -= W^* W, invert the trailing half, N12 = -N11 W N22.
+// The factor itself is never formed, and no triangular system is solved:
+// every step above the innermost blocks is a product with K = half the width.
 template <class T>
-static void chol_row_rec(cudaStream_t st, int r0, int r1, int j0, int j1, T* Z, int ldz, long long sZ, const T* Rinv,
-                         long long sR, int batch) {
-  const int w = r1 - r0;
-  const T one = from_re<T>(1.0), mone = from_re<T>(-1.0), zer = zero<T>();
-  T* Zr = Z + r0 + (long long)j0 * ldz;
-  if (w <= NB_CHOL) {
-    GemmArgs<T> g;
-    g.batch = batch;
-    g.m = w; g.n = j1 - j0; g.k = w; g.opA = OP_C; g.opB = OP_N;
-    g.A = Rinv + (long long)r0 * NB_CHOL; g.lda = NB_CHOL; g.sA = sR;
-    g.B = Zr; g.ldb = ldz; g.sB = sZ;
-    g.C = Zr; g.ldc = ldz; g.sC = sZ;
-    g.site = GS_CHOL_ROW;
-    g.alpha = one; g.beta = zer; g.kflags = K_TO_ROW;
-    gemm(g, st);
-    return;
-  }
-  const int rm = r0 + ceil_div(w / 2, NB_CHOL) * NB_CHOL;
-  chol_row_rec(st, r0, rm, j0, j1, Z, ldz, sZ, Rinv, sR, batch);
-  GemmArgs<T> g;  // Z[rm:r1, j0:j1] -= R[r0:rm, rm:r1]^* X[r0:rm, j0:j1]
-  g.batch = batch;
-  g.m = r1 - rm; g.n = j1 - j0; g.k = rm - r0; g.opA = OP_C; g.opB = OP_N;
-  g.A = Z + r0 + (long long)rm * ldz; g.lda = ldz; g.sA = sZ;
-  g.B = Zr; g.ldb = ldz; g.sB = sZ;
-  T* Z2 = Z + rm + (long long)j0 * ldz;
-  g.Cin = Z2; g.ldcin = ldz; g.sCin = sZ;
-  g.C = Z2; g.ldc = ldz; g.sC = sZ;
-  g.site = GS_CHOL_ROW;
-  g.alpha = mone; g.beta = one;
-  gemm(g, st);
-  chol_row_rec(st, rm, r1, j0, j1, Z, ldz, sZ, Rinv, sR, batch);
-}
-
-// Recursive Cholesky Z = R^* R on [c0, c1): factor the leading half, solve
-// its rows R12 = R11^{-*} Z12, update Z22 -= R12^* R12 (one product with K =
-// half the width), factor Z22.  Leaves of NB_CHOL columns factor and invert
-// the diagonal block.
-template <class T>
-static void chol_rec(cudaStream_t st, int n, int c0, int c1, T* Z, int ldz, long long sZ, T* Rinv, long long sR,
-                     int* info, int batch) {
+static void chol_inv_rec(cudaStream_t st, Arena& ar, int c0, int c1, T* Z, int ldz, long long sZ, T* N, int ldn,
+                         long long sN, int batch) {
+  constexpr int NB = chol_nb<T>();
   const int w = c1 - c0;
-  if (w <= NB_CHOL) {
-    potrf_inv<T>(st, n, Z, ldz, sZ, c0, w, Rinv + (long long)c0 * NB_CHOL, NB_CHOL, sR, info, batch);
+  if (w <= NB) {
+    chol_inv_block<T>(st, w, Z + c0 + (long long)c0 * ldz, ldz, sZ, N + c0 + (long long)c0 * ldn, ldn, sN, batch);
     return;
   }
-  const int mid = c0 + ceil_div(w / 2, NB_CHOL) * NB_CHOL;
-  chol_rec(st, n, c0, mid, Z, ldz, sZ, Rinv, sR, info, batch);
-  chol_row_rec(st, c0, mid, mid, c1, Z, ldz, sZ, Rinv, sR, batch);
-  GemmArgs<T> g;  // Z22 -= R12^* R12  (tiles touching the upper triangle)
-  g.batch = batch;
-  g.m = c1 - mid; g.n = c1 - mid; g.k = mid - c0; g.opA = OP_C; g.opB = OP_N;
-  T* R12 = Z + c0 + (long long)mid * ldz;
-  g.A = R12; g.lda = ldz; g.sA = sZ;
-  g.B = R12; g.ldb = ldz; g.sB = sZ;
-  T* Z22 = Z + mid + (long long)mid * ldz;
-  g.Cin = Z22; g.ldcin = ldz; g.sCin = sZ;
-  g.C = Z22; g.ldc = ldz; g.sC = sZ;
-  g.site = GS_CHOL_TRAIL;
-  g.alpha = from_re<T>(-1.0); g.beta = from_re<T>(1.0); g.uplo = 1;
-  gemm(g, st);
-  chol_rec(st, n, mid, c1, Z, ldz, sZ, Rinv, sR, info, batch);
-}
-
-template <class T>
-void cholesky(cudaStream_t st, int n, T* Z, int ldz, long long sZ, T* Rinv, long long sR, int* info, int batch) {
-  ZCSD_CUDA(cudaMemsetAsync(info, 0, sizeof(int) * batch, st));
-  chol_rec(st, n, 0, n, Z, ldz, sZ, Rinv, sR, info, batch);
-}
-
-// Recursive right-side triangular solves on column ranges [c0, c1) aligned to
-// NB_CHOL: Y R = X splits R = [R11 R12; 0 R22] into Y1 = X1 R11^{-1},
-// X2 -= Y1 R12, Y2 = X2 R22^{-1}; leaves multiply by the inverted diagonal
-// blocks.  The off-diagonal updates are n x (w/2) x (w/2) products.
-template <class T>
-static void trsm_fwd_rec(cudaStream_t st, int n, int c0, int c1, T* Yt, int ldt, long long sT, const T* Z, int ldz,
-                         long long sZ, const T* Rinv, long long sR, T* Tmp, int batch) {
-  const int w = c1 - c0;
+  const int mid = c0 + ceil_div(w / 2, NB) * NB, w1 = mid - c0, w2 = c1 - mid;
   const T one = from_re<T>(1.0), mone = from_re<T>(-1.0), zer = zero<T>();
-  if (w <= NB_CHOL) {
-    axpby<T>(st, n, w, 1.0, Yt + (long long)c0 * ldt, ldt, sT, 0.0, Tmp, n, (long long)n * NB_CHOL, batch);
-    GemmArgs<T> g;  // Y[:, c0:c1] = X[:, c0:c1] R_kk^{-1}
-    g.batch = batch;
-    g.m = n; g.n = w; g.k = w; g.opA = OP_N; g.opB = OP_N;
-    g.A = Tmp; g.lda = n; g.sA = (long long)n * NB_CHOL;
-    g.B = Rinv + (long long)c0 * NB_CHOL; g.ldb = NB_CHOL; g.sB = sR;
-    g.C = Yt + (long long)c0 * ldt; g.ldc = ldt; g.sC = sT;
-    g.alpha = one; g.beta = zer; g.kflags = K_TO_COL; g.site = GS_TRSM_F_DIAG;
-    gemm(g, st);
-    return;
-  }
-  const int mid = c0 + ceil_div(w / 2, NB_CHOL) * NB_CHOL;
-  trsm_fwd_rec(st, n, c0, mid, Yt, ldt, sT, Z, ldz, sZ, Rinv, sR, Tmp, batch);
-  GemmArgs<T> g;  // X2 -= Y1 R12
-  g.batch = batch;
-  g.m = n; g.n = c1 - mid; g.k = mid - c0; g.opA = OP_N; g.opB = OP_N;
-  g.A = Yt + (long long)c0 * ldt; g.lda = ldt; g.sA = sT;
-  g.B = Z + c0 + (long long)mid * ldz; g.ldb = ldz; g.sB = sZ;
-  g.Cin = Yt + (long long)mid * ldt; g.ldcin = ldt; g.sCin = sT;
-  g.C = Yt + (long long)mid * ldt; g.ldc = ldt; g.sC = sT;
-  g.alpha = mone; g.beta = one; g.site = GS_TRSM_F_UPD;
-  gemm(g, st);
-  trsm_fwd_rec(st, n, mid, c1, Yt, ldt, sT, Z, ldz, sZ, Rinv, sR, Tmp, batch);
-}
-
-// T R^* = Y with R^* lower triangular: T2 = Y2 R22^{-*}, Y1 -= T2 R12^*, T1 = Y1 R11^{-*}.
-template <class T>
-static void trsm_bwd_rec(cudaStream_t st, int n, int c0, int c1, T* Tt, int ldt, long long sT, const T* Z, int ldz,
-                         long long sZ, const T* Rinv, long long sR, T* Tmp, int batch) {
-  const int w = c1 - c0;
-  const T one = from_re<T>(1.0), mone = from_re<T>(-1.0), zer = zero<T>();
-  if (w <= NB_CHOL) {
-    axpby<T>(st, n, w, 1.0, Tt + (long long)c0 * ldt, ldt, sT, 0.0, Tmp, n, (long long)n * NB_CHOL, batch);
-    GemmArgs<T> g;  // T[:, c0:c1] = Y[:, c0:c1] R_kk^{-*}
-    g.batch = batch;
-    g.m = n; g.n = w; g.k = w; g.opA = OP_N; g.opB = OP_C;
-    g.A = Tmp; g.lda = n; g.sA = (long long)n * NB_CHOL;
-    g.B = Rinv + (long long)c0 * NB_CHOL; g.ldb = NB_CHOL; g.sB = sR;
-    g.C = Tt + (long long)c0 * ldt; g.ldc = ldt; g.sC = sT;
-    g.alpha = one; g.beta = zer; g.kflags = K_FROM_COL; g.site = GS_TRSM_B_DIAG;
-    gemm(g, st);
-    return;
-  }
-  const int mid = c0 + ceil_div(w / 2, NB_CHOL) * NB_CHOL;
-  trsm_bwd_rec(st, n, mid, c1, Tt, ldt, sT, Z, ldz, sZ, Rinv, sR, Tmp, batch);
-  GemmArgs<T> g;  // Y1 -= T2 R12^*
-  g.batch = batch;
-  g.m = n; g.n = mid - c0; g.k = c1 - mid; g.opA = OP_N; g.opB = OP_C;
-  g.A = Tt + (long long)mid * ldt; g.lda = ldt; g.sA = sT;
-  g.B = Z + c0 + (long long)mid * ldz; g.ldb = ldz; g.sB = sZ;
-  g.Cin = Tt + (long long)c0 * ldt; g.ldcin = ldt; g.sCin = sT;
-  g.C = Tt + (long long)c0 * ldt; g.ldc = ldt; g.sC = sT;
-  g.alpha = mone; g.beta = one; g.site = GS_TRSM_B_UPD;
-  gemm(g, st);
-  trsm_bwd_rec(st, n, c0, mid, Tt, ldt, sT, Z, ldz, sZ, Rinv, sR, Tmp, batch);
-}
-
-template <class T>
-void trsm_pair(cudaStream_t st, Arena& ar, int n, const T* X, int ldx, long long sX, int xdiv, const T* Z, int ldz,
-               long long sZ, const T* Rinv, long long sR, T* Yt, T* Tt, int ldt, long long sT, int batch) {
+  chol_inv_rec(st, ar, c0, mid, Z, ldz, sZ, N, ldn, sN, batch);
   const size_t mk = ar.mark();
-  T* Tmp = ar.get<T>((size_t)n * NB_CHOL * batch);
-  // Yt = X (problem b reads X_{b / xdiv}), then solve in place
-  const int P = batch / xdiv;
-  for (int j = 0; j < xdiv; ++j)
-    axpby<T>(st, n, n, 1.0, X, ldx, sX, 0.0, Yt + (long long)j * sT, ldt, sT * xdiv, P);
-  trsm_fwd_rec(st, n, 0, n, Yt, ldt, sT, Z, ldz, sZ, Rinv, sR, Tmp, batch);
-  axpby<T>(st, n, n, 1.0, Yt, ldt, sT, 0.0, Tt, ldt, sT, batch);
-  trsm_bwd_rec(st, n, 0, n, Tt, ldt, sT, Z, ldz, sZ, Rinv, sR, Tmp, batch);
+  const long long sW = (long long)w1 * w2;
+  T* W = ar.get<T>((size_t)sW * batch);
+  T* N11 = N + c0 + (long long)c0 * ldn;
+  GemmArgs<T> g;  // W = N11^* Z12
+  g.batch = batch;
+  g.m = w1; g.n = w2; g.k = w1; g.opA = OP_C; g.opB = OP_N; g.kflags = K_TO_ROW;
+  g.A = N11; g.lda = ldn; g.sA = sN;
+  g.B = Z + c0 + (long long)mid * ldz; g.ldb = ldz; g.sB = sZ;
+  g.C = W; g.ldc = w1; g.sC = sW;
+  g.alpha = one; g.beta = zer; g.site = GS_CHOL_INV;
+  gemm(g, st);
+  GemmArgs<T> h;  // Z22 -= W^* W (tiles touching the upper triangle)
+  h.batch = batch;
+  h.m = w2; h.n = w2; h.k = w1; h.opA = OP_C; h.opB = OP_N; h.uplo = 1;
+  h.A = W; h.lda = w1; h.sA = sW;
+  h.B = W; h.ldb = w1; h.sB = sW;
+  T* Z22 = Z + mid + (long long)mid * ldz;
+  h.Cin = Z22; h.ldcin = ldz; h.sCin = sZ;
+  h.C = Z22; h.ldc = ldz; h.sC = sZ;
+  h.alpha = mone; h.beta = one; h.site = GS_CHOL_TRAIL;
+  gemm(h, st);
+  chol_inv_rec(st, ar, mid, c1, Z, ldz, sZ, N, ldn, sN, batch);
+  T* V = ar.get<T>((size_t)sW * batch);
+  GemmArgs<T> v;  // V = W N22
+  v.batch = batch;
+  v.m = w1; v.n = w2; v.k = w2; v.opA = OP_N; v.opB = OP_N; v.kflags = K_TO_COL;
+  v.A = W; v.lda = w1; v.sA = sW;
+  v.B = N + mid + (long long)mid * ldn; v.ldb = ldn; v.sB = sN;
+  v.C = V; v.ldc = w1; v.sC = sW;
+  v.alpha = one; v.beta = zer; v.site = GS_CHOL_INV;
+  gemm(v, st);
+  GemmArgs<T> u;  // N12 = -N11 V
+  u.batch = batch;
+  u.m = w1; u.n = w2; u.k = w1; u.opA = OP_N; u.opB = OP_N; u.kflags = K_FROM_ROW;
+  u.A = N11; u.lda = ldn; u.sA = sN;
+  u.B = V; u.ldb = w1; u.sB = sW;
+  u.C = N + c0 + (long long)mid * ldn; u.ldc = ldn; u.sC = sN;
+  u.alpha = mone; u.beta = zer; u.site = GS_CHOL_INV;
+  gemm(u, st);
   ar.release(mk);
+}
+
+template <class T>
+void chol_inverse(cudaStream_t st, Arena& ar, int n, T* Z, int ldz, long long sZ, T* N, int ldn, long long sN,
+                  int batch) {
+  chol_inv_rec<T>(st, ar, 0, n, Z, ldz, sZ, N, ldn, sN, batch);
+}
+
+template <class T>
+void gemm_terms(GemmArgs<T> g, cudaStream_t st) {
+  if constexpr (std::is_same<T, z64>::value) {
+    GemmArgs<T> one = g;
+    one.nsum = 1;
+    if (g.nsum > 1 && tc_will_handle_complex(one)) {
+      for (int j = 0; j < g.nsum; ++j) {
+        one.A = g.A + j * g.sAj;
+        one.B = g.B + j * g.sBj;
+        one.alpha = scal(g.w[j], g.alpha);
+        if (j > 0) {
+          one.Cin = g.C; one.ldcin = g.ldc; one.sCin = g.sC;
+          one.beta = from_re<T>(1.0);
+        }
+        gemm(one, st);
+      }
+      return;
+    }
+  }
+  gemm(g, st);
 }
 
 #define ZCSD_INST_L(T)                                                                                          \
   template QRStore<T> qr_alloc<T>(Arena&, int, int, int, int);                                                  \
   template void qr_factor<T>(cudaStream_t, Arena&, QRStore<T>&, T*, int, long long);                            \
   template void qr_form_q<T>(cudaStream_t, Arena&, const QRStore<T>&, T*, int, long long);                      \
-  template void cholesky<T>(cudaStream_t, int, T*, int, long long, T*, long long, int*, int);                   \
-  template void trsm_pair<T>(cudaStream_t, Arena&, int, const T*, int, long long, int, const T*, int, long long, \
-                             const T*, long long, T*, T*, int, long long, int);
+  template void chol_inverse<T>(cudaStream_t, Arena&, int, T*, int, long long, T*, int, long long, int);         \
+  template void gemm_terms<T>(GemmArgs<T>, cudaStream_t);
 
 ZCSD_INST_L(double)
 ZCSD_INST_L(z64)

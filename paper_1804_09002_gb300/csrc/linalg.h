@@ -10,7 +10,6 @@ namespace zcsd {
 
 constexpr int NB_QR = 32;    // Householder panel width
 constexpr int NB_OUT = 128;  // outer block of the two-level blocked QR
-constexpr int NB_CHOL = 64;  // Cholesky / TRSM block size
 constexpr int LEAF = 1024;   // Zolo-eig leaf size, default (leaf.cu: a 1024-row leaf is faster than one split of it)
 constexpr int LEAF_MAX = 1024;  // largest leaf size a context may set
 
@@ -48,7 +47,6 @@ struct HostScalars {
 template <class T>
 struct QRStore {
   int m = 0, n = 0, band = 0, batch = 0, npan = 0, ldy = 0, nbo = 0;
-  int xrows = 0;    // rows [0, xrows) form the dense block X of a stacked [X; sqrt(c) I] (0: not stacked)
   T* Y = nullptr;  // per problem: npan outer blocks of ldy x nbo (nbo = min(NB_OUT, n rounded up to 32))
   T* Tf = nullptr; // per problem: npan blocks of nbo x nbo
   long long sY = 0, sT = 0;
@@ -59,16 +57,16 @@ template <class T> void qr_factor(cudaStream_t st, Arena& ar, QRStore<T>& q, T* 
 // E_b = Q_b [I; 0] (m x n, ld lde, stride sE)
 template <class T> void qr_form_q(cudaStream_t st, Arena& ar, const QRStore<T>& q, T* E, int lde, long long sE);
 
-// ---- upper Cholesky R^* R = Z_b (in place, upper triangle) of `batch` n x n
-// matrices; Rinv receives the inverses of the NB_CHOL diagonal blocks
-// (per problem NB_CHOL x n, block k at column k*NB_CHOL).  info[b] != 0 on a
-// non-positive pivot.
+// ---- N_b = R_b^{-1}, the inverse of the upper Cholesky factor R^* R = Z_b, of
+// `batch` n x n matrices.  Z's upper triangle is overwritten; N must be zero
+// below its diagonal on entry (it stays so).
 template <class T>
-void cholesky(cudaStream_t st, int n, T* Z, int ldz, long long sZ, T* Rinv, long long sR, int* info, int batch);
+void chol_inverse(cudaStream_t st, Arena& ar, int n, T* Z, int ldz, long long sZ, T* N, int ldn, long long sN,
+                  int batch);
 
-// ---- Tt_b = X_{b / xdiv} (R_b^* R_b)^{-1}: Yt = X R^{-1}, then Tt = Yt R^{-*}.
+// ---- C = alpha sum_j w_j op(A_j) op(B_j) + beta Cin, as gemm(); complex sums
+// go term by term where that lets the tensor cores take them.
 template <class T>
-void trsm_pair(cudaStream_t st, Arena& ar, int n, const T* X, int ldx, long long sX, int xdiv, const T* Z, int ldz,
-               long long sZ, const T* Rinv, long long sR, T* Yt, T* Tt, int ldt, long long sT, int batch);
+void gemm_terms(GemmArgs<T> g, cudaStream_t st);
 
 }  // namespace zcsd

@@ -23,8 +23,8 @@ constexpr int MAX_SUM = 16;
 // Call sites of the GEMM, for per-site kernel accounting.
 enum GemmSite {
   GS_OTHER = 0, GS_QR_W, GS_QR_W2, GS_QR_UPD, GS_FQ_W, GS_FQ_W2, GS_FQ_UPD, GS_ZOLO_COMBINE, GS_GRAM,
-  GS_CHOL_ROW, GS_CHOL_TRAIL, GS_TRSM_F_UPD, GS_TRSM_F_DIAG, GS_TRSM_B_UPD, GS_TRSM_B_DIAG, GS_H, GS_ORTH,
-  GS_EIG, GS_ASSEMBLY, GS_ALG2, GS_TMERGE, GS_QR_UPD_X, GS_GRAD, GS_SITES
+  GS_CHOL_INV, GS_CHOL_TRAIL, GS_INV_SUM, GS_ZOLO_Q, GS_INV_APPLY, GS_ZOLO_GRAM2, GS_H, GS_ORTH,
+  GS_EIG, GS_ASSEMBLY, GS_ALG2, GS_TMERGE, GS_ZOLO_POLISH, GS_GRAD, GS_SITES
 };
 
 template <class T>
@@ -67,13 +67,17 @@ template <class T> void sum_parts(cudaStream_t st, int m, int n, T* X, int ldx, 
 // Y_j = X + shift_j I for j < nterms (shifts on device or by value), Y_j at stride sY
 template <class T> void shift_terms(cudaStream_t st, int n, const T* X, int ldx, long long sXb,
                                     const double* shifts, int nterms, T* Y, int ldy, long long sY, int batch);
-// M_j = [X; sqrt(c_j) I] (2n x n, ld = ldm), for j < nterms of each of `batch` X's
-template <class T> void stack_terms(cudaStream_t st, int n, const T* X, int ldx, long long sXb,
-                                    const double* sqrtc, int nterms, T* M, int ldm, long long sM, int batch);
-// X2 = mhat (X1 + sum_j a_j T_j)
-template <class T> void sum_terms(cudaStream_t st, int n, double mhat, const T* X1, int ldx, long long sXb,
-                                  const double* a, int nterms, const T* Tm, int ldt, long long sT,
-                                  T* X2, int ldx2, long long sX2b, int batch);
+// Z_b = alpha X_b + beta I
+template <class T> void scale_shift(cudaStream_t st, int n, double alpha, const T* X, int ldx, long long sX,
+                                    double beta, T* Z, int ldz, long long sZ, int batch);
+// X_{b nterms + j} *= s_j (m x n)
+template <class T> void scale_terms(cudaStream_t st, int m, int n, const double* s, int nterms, T* X, int ldx,
+                                    long long sX, int batch);
+// E = X - I from the upper triangle of the Hermitian X, both triangles
+template <class T> void minus_eye(cudaStream_t st, int n, const T* X, int ldx, long long sX, T* E, int lde,
+                                  long long sE, int batch);
+// the lower triangle of the Hermitian X from its upper one
+template <class T> void mirror(cudaStream_t st, int n, T* X, int ldx, long long sX, int batch);
 // H = (Y + Y^*)/2 (in place allowed)
 template <class T> void symmetrize(cudaStream_t st, int n, const T* Y, int ldy, long long sY, T* H, int ldh,
                                    long long sH, int batch);
@@ -110,9 +114,10 @@ template <class T> void randn(cudaStream_t st, int m, int n, T* X, int ldx, unsi
 // tau, and the nb x nb upper triangular T of Q = I - V T V^* (ld = nbmax).
 template <class T> void qr_panel(cudaStream_t st, int m, int n, int band, T* M, int ldm, long long sM,
                                  int k0, int nb, T* Y, int ldy, long long sY, T* Tf, long long sT, int batch);
-// Upper Cholesky R^* R = A_kk of the nb x nb diagonal block at (k0, k0) and
-// its inverse R^{-1} (written to Rinv, ld = nb_ld, zeros below the diagonal).
-// info[b] is set to (k0 + j + 1) at the first non-positive pivot.
-template <class T> void potrf_inv(cudaStream_t st, int n, T* A, int lda, long long sA, int k0, int nb,
-                                  T* Rinv, int ldr, long long sR, int* info, int batch);
+// N = R^{-1} (upper triangular; only its upper triangle is written) of the
+// upper Cholesky factor R^* R = Z of nb x nb blocks, nb <= chol_nb, from Z's
+// upper triangle; NaN where Z is not positive definite.
+template <class T> __host__ __device__ constexpr int chol_nb() { return sizeof(T) == 8 ? 64 : 32; }
+template <class T> void chol_inv_block(cudaStream_t st, int nb, const T* Z, int ldz, long long sZ, T* N, int ldn,
+                                       long long sN, int batch);
 }  // namespace zcsd

@@ -98,14 +98,179 @@ void d2h(Ctx& cx, void* dst, const void* src, size_t bytes) {
 
 // ---------------------------------------------------------------- Zolo-pd
 
-// W_p = Zolo-pd polar factor of X0_p (p < P), X0 with ||X0_p||_2 <= 1 (ld n,
-// stride n*n).  W may alias nothing else.  Section 5: iterates
-// X_{k+1} = M (X_k + sum_j a_j X_k (X_k^* X_k + c_{2j-1} I)^{-1}); the first
-// iteration in QR form (X (X^*X + cI)^{-1} = Q1 Q2^* / sqrt(c) for
-// [X; sqrt(c) I] = [Q1; Q2] R), later ones in Cholesky form.
+// First Zolo-pd iteration: X_new = mhat X + sum_j (mhat a_j / sqrt(c_j)) Q1_j
+// Q2_j^*, [Q1_j; Q2_j] an orthonormal basis of [X; sqrt(c_j) I] (X (X^* X + c
+// I)^{-1} = Q1 Q2^* / sqrt(c); any basis gives the same term, so the QR factor
+// of Section 5 is not needed).  The shifts c_j are about 4700 apart, which a
+// chain of Cholesky factorizations uses:
+//   * the largest, 8.5e-4: X^* X + c I has condition number 1200; with N its
+//     inverse Cholesky factor, Q1 = X N and Q2 = sqrt(c) N;
+//   * the basis of term j + 1 preconditions term j: the columns of
+//     [Q1; sqrt(rho) Q2], rho = c_j / c_{j+1}, span [X; sqrt(c_j) I], and their
+//     Gram matrix rho I + (1 - rho) Q1^* Q1 has condition number 1 / rho; its
+//     inverse Cholesky factor orthonormalises them.  It is positive definite
+//     for every X, so there is no pivot to check.
+// Each step leaves a departure E = Q1^* Q1 + Q2^* Q2 - I of order u / rho,
+// which does not grow along the chain; to first order the term of the exact
+// basis is (Q1 - Q1 E) Q2^*, one more product.  The result is as accurate as
+// with Householder factorizations of the stacked matrices (backward error 14 u
+// against 13 u, at any sigma_min) and all but the 64-column blocks are
+// products with large K: the Householder panels took a fifth of a
+// decomposition and their updates, with K = 128, most of the rest (polar of
+// n = 2048 130 -> 86 ms, a complex n = 512 decomposition 155 -> 113 ms).
 template <class T>
-void zolo_pd(Ctx& cx, Arena& ar, int n, int P, const T* X0, T* W, PolarDiag* pd, int stop_after,
-             int reduced_slices, bool sync_free) {
+static void zolo_first(cudaStream_t st, Arena& ar, const Plan& pl, int n, int P, const T* X, T* Xn) {
+  const int r = pl.r[0];
+  const long long nn = (long long)n * n, sM = 2 * nn;  // E_j = [Q1; Q2], ld 2n
+  const int m2 = 2 * n;
+  const T one = from_re<T>(1.0), mone = from_re<T>(-1.0), zer = zero<T>();
+  const size_t mk = ar.mark();
+  T* E = ar.get<T>(sM * P * r);   // Q2 as N, the accumulated inverse factors: scaled by sqrt(c_j) at the end
+  T* G = ar.get<T>(nn * P * r);   // Gram matrices Q1^* Q1
+  T* Z = ar.get<T>(nn * P);
+  T* N = ar.get<T>(nn * P);
+  ZCSD_CUDA(cudaMemsetAsync(N, 0, sizeof(T) * nn * P, st));
+  auto gram = [&](const T* A, int lda, long long sA, T* C, long long sC) {
+    GemmArgs<T> g;
+    g.batch = P;
+    g.m = n; g.n = n; g.k = n; g.opA = OP_C; g.opB = OP_N; g.uplo = 1;
+    g.A = A; g.lda = lda; g.sA = sA;
+    g.B = A; g.ldb = lda; g.sB = sA;
+    g.C = C; g.ldc = n; g.sC = sC;
+    g.alpha = one; g.beta = zer; g.site = GS_GRAM;
+    gemm(g, st);
+  };
+  // rows of [Q1; Q2] times N: together while a launch costs more than the
+  // zeros of Q2, apart above
+  const bool together = n <= 256;
+  for (int j = r - 1; j >= 0; --j) {
+    T* Ej = E + j * sM;
+    const bool first = j == r - 1;
+    const double c = pl.c[0][2 * j], rho = first ? 1.0 : c / pl.c[0][2 * (j + 1)];
+    if (first) {
+      gram(X, n, nn, G + j * nn, nn * r);
+      scale_shift<T>(st, n, 1.0, G + j * nn, n, nn * r, c, Z, n, nn, P);
+    } else {
+      scale_shift<T>(st, n, 1.0 - rho, G + (j + 1) * nn, n, nn * r, rho, Z, n, nn, P);
+    }
+    chol_inverse<T>(st, ar, n, Z, n, nn, N, n, nn, P);
+    GemmArgs<T> g;
+    g.batch = P;
+    g.m = (!first && together) ? m2 : n; g.n = n; g.k = n; g.opA = OP_N; g.opB = OP_N; g.kflags = K_TO_COL;
+    if (first) { g.A = X; g.lda = n; g.sA = nn; }
+    else { g.A = Ej + sM; g.lda = m2; g.sA = sM * r; }
+    g.B = N; g.ldb = n; g.sB = nn;
+    g.C = Ej; g.ldc = m2; g.sC = sM * r;
+    g.alpha = one; g.beta = zer; g.site = GS_ZOLO_Q;
+    gemm(g, st);
+    if (first) {
+      axpby<T>(st, n, n, 1.0, N, n, nn, 0.0, Ej + n, m2, sM * r, P);
+    } else if (!together) {
+      g.A += n;
+      g.C += n;
+      g.kflags = K_TO_COL | K_FROM_ROW;
+      gemm(g, st);
+    }
+    gram(Ej, m2, sM * r, G + j * nn, nn * r);
+  }
+  scale_terms<T>(st, n, n, pl.sqrtc[0], r, E + n, m2, sM, P);
+  {
+    GemmArgs<T> g;  // Q1^* Q1 + Q2^* Q2
+    g.batch = P * r;
+    g.m = n; g.n = n; g.k = n; g.opA = OP_C; g.opB = OP_N; g.uplo = 1; g.kflags = K_TO_ROW | K_TO_COL;
+    g.A = E + n; g.lda = m2; g.sA = sM;
+    g.B = E + n; g.ldb = m2; g.sB = sM;
+    g.Cin = G; g.ldcin = n; g.sCin = nn;
+    g.C = G; g.ldc = n; g.sC = nn;
+    g.alpha = one; g.beta = one; g.site = GS_ZOLO_GRAM2;
+    gemm(g, st);
+  }
+  T* F = ar.get<T>(nn * P * r);
+  minus_eye<T>(st, n, G, n, nn, F, n, nn, P * r);
+  T* Y = G;  // the Gram matrices are done with
+  {
+    GemmArgs<T> g;  // Y = Q1 - Q1 (Q1^* Q1 + Q2^* Q2 - I)
+    g.batch = P * r;
+    g.m = n; g.n = n; g.k = n; g.opA = OP_N; g.opB = OP_N;
+    g.A = E; g.lda = m2; g.sA = sM;
+    g.B = F; g.ldb = n; g.sB = nn;
+    g.Cin = E; g.ldcin = m2; g.sCin = sM;
+    g.C = Y; g.ldc = n; g.sC = nn;
+    g.alpha = mone; g.beta = one; g.site = GS_ZOLO_POLISH;
+    gemm(g, st);
+  }
+  {
+    GemmArgs<T> g;  // X_new (Q2 upper triangular)
+    g.batch = P;
+    g.m = n; g.n = n; g.k = n; g.opA = OP_N; g.opB = OP_C; g.kflags = K_FROM_COL;
+    g.A = Y; g.lda = n; g.sA = nn * r; g.sAj = nn;
+    g.B = E + n; g.ldb = m2; g.sB = sM * r; g.sBj = sM;
+    g.nsum = r;
+    for (int j = 0; j < r; ++j) g.w[j] = pl.w[0][j];
+    g.Cin = X; g.ldcin = n; g.sCin = nn;
+    g.C = Xn; g.ldc = n; g.sC = nn;
+    g.alpha = one; g.beta = from_re<T>(pl.mhat[0]); g.site = GS_ZOLO_COMBINE;
+    gemm_terms(g, st);
+  }
+  ar.release(mk);
+}
+
+// Later iterations, Cholesky form: X_new = mhat (X + X sum_j a_j Z_j^{-1}),
+// Z_j = X^* X + c_j I = R_j^* R_j.  X's singular values lie in [l_s, 1], so the
+// Z_j are well conditioned and their inverses N_j N_j^*, N_j = R_j^{-1}, are
+// summed before they meet X: one symmetric sum of triangular products and one
+// product with X in place of two triangular solves per term.
+template <class T>
+static void zolo_next(cudaStream_t st, Arena& ar, const Plan& pl, int s, int n, int P, const T* X, T* Xn) {
+  const int r = pl.r[s];
+  const long long nn = (long long)n * n;
+  const T one = from_re<T>(1.0), zer = zero<T>();
+  const size_t mk = ar.mark();
+  T* G = ar.get<T>(nn * P);
+  T* Z = ar.get<T>(nn * P * r);
+  T* N = ar.get<T>(nn * P * r);
+  ZCSD_CUDA(cudaMemsetAsync(N, 0, sizeof(T) * nn * P * r, st));
+  GemmArgs<T> g;
+  g.batch = P;
+  g.m = n; g.n = n; g.k = n; g.opA = OP_C; g.opB = OP_N; g.uplo = 1;
+  g.A = X; g.lda = n; g.sA = nn;
+  g.B = X; g.ldb = n; g.sB = nn;
+  g.C = G; g.ldc = n; g.sC = nn;
+  g.alpha = one; g.beta = zer; g.site = GS_GRAM;
+  gemm(g, st);
+  double shifts[R_MAX];
+  for (int j = 0; j < r; ++j) shifts[j] = pl.c[s][2 * j];
+  shift_terms<T>(st, n, G, n, nn, shifts, r, Z, n, nn, P);
+  chol_inverse<T>(st, ar, n, Z, n, nn, N, n, nn, P * r);
+  GemmArgs<T> h;  // G = sum_j a_j N_j N_j^*
+  h.batch = P;
+  h.m = n; h.n = n; h.k = n; h.opA = OP_N; h.opB = OP_C; h.uplo = 1; h.kflags = K_FROM_ROW | K_FROM_COL;
+  h.A = N; h.lda = n; h.sA = nn * r; h.sAj = nn;
+  h.B = N; h.ldb = n; h.sB = nn * r; h.sBj = nn;
+  h.nsum = r;
+  for (int j = 0; j < r; ++j) h.w[j] = pl.a[s][j];
+  h.C = G; h.ldc = n; h.sC = nn;
+  h.alpha = one; h.beta = zer; h.site = GS_INV_SUM;
+  gemm_terms(h, st);
+  mirror<T>(st, n, G, n, nn, P);
+  GemmArgs<T> x;
+  x.batch = P;
+  x.m = n; x.n = n; x.k = n; x.opA = OP_N; x.opB = OP_N;
+  x.A = X; x.lda = n; x.sA = nn;
+  x.B = G; x.ldb = n; x.sB = nn;
+  x.Cin = X; x.ldcin = n; x.sCin = nn;
+  x.C = Xn; x.ldc = n; x.sC = nn;
+  x.alpha = from_re<T>(pl.mhat[s]); x.beta = from_re<T>(pl.mhat[s]); x.site = GS_INV_APPLY;
+  gemm(x, st);
+  ar.release(mk);
+}
+
+// W_p = Zolo-pd polar factor of X0_p (p < P), X0 with ||X0_p||_2 <= 1 (ld n,
+// stride n*n).  W may alias X0.  Section 5: iterates
+// X_{k+1} = M (X_k + sum_j a_j X_k (X_k^* X_k + c_{2j-1} I)^{-1}); the first
+// iteration from orthonormal bases, later ones in Cholesky form.
+template <class T>
+void zolo_pd(Ctx& cx, Arena& ar, int n, int P, const T* X0, T* W, PolarDiag* pd, int stop_after, int reduced_slices) {
   cudaStream_t st = cx.stream;
   const Plan& pl = get_plan(cx);
   const int steps = (stop_after > 0) ? std::min(stop_after, pl.steps) : pl.steps;
@@ -113,110 +278,44 @@ void zolo_pd(Ctx& cx, Arena& ar, int n, int P, const T* X0, T* W, PolarDiag* pd,
   const size_t mk = ar.mark();
   T* Xa = ar.get<T>(nn * P);
   T* Xb = ar.get<T>(nn * P);
-  axpby<T>(st, n, n, 1.0, X0, n, nn, 0.0, Xa, n, nn, P);
-  T* X = Xa;
-  T* Xn = Xb;
-  const T one = from_re<T>(1.0), mone = from_re<T>(-1.0), zer = zero<T>();
+  const T* X = X0;
   for (int s = 0; s < steps; ++s) {
-    const int r = pl.r[s];
-    bool use_qr = (s == 0);
+    T* Xn = s + 1 == steps && X != W && X0 != W ? W : (X == Xa ? Xb : Xa);
     if (pd) pd->iters += 1;
-    for (int attempt = 0; attempt < 2; ++attempt) {
-      const size_t mk2 = ar.mark();
-      if (use_qr) {
-        // ---- QR form on the stacked [X; sqrt(c_{2j-1}) I], 2n x n, P*r problems
-        const int m2 = 2 * n;
-        const long long sM = (long long)m2 * n;
-        T* M = ar.get<T>(sM * P * r);
-        T* E = ar.get<T>(sM * P * r);
-        stack_terms<T>(st, n, X, n, nn, pl.sqrtc[s], r, M, m2, sM, P);
-        QRStore<T> q = qr_alloc<T>(ar, m2, n, n + 1, P * r);
-        q.xrows = n;
-        qr_factor<T>(st, ar, q, M, m2, sM);
-        qr_form_q<T>(st, ar, q, E, m2, sM);
-        // X_new = mhat X + sum_j (mhat a_j / sqrt(c_j)) Q1_j Q2_j^*   (Q2 upper triangular)
-        GemmArgs<T> g;
-        g.batch = P;
-        g.m = n; g.n = n; g.k = n; g.opA = OP_N; g.opB = OP_C;
-        g.A = E; g.lda = m2; g.sA = sM * r; g.sAj = sM;
-        g.B = E + n; g.ldb = m2; g.sB = sM * r; g.sBj = sM;
-        g.nsum = r;
-        for (int j = 0; j < r; ++j) g.w[j] = pl.w[s][j];
-        g.Cin = X; g.ldcin = n; g.sCin = nn;
-        g.C = Xn; g.ldc = n; g.sC = nn;
-        g.alpha = one; g.beta = from_re<T>(pl.mhat[s]);
-        g.kflags = K_FROM_COL;
-        g.site = GS_ZOLO_COMBINE;
-        gemm(g, st);
-        ar.release(mk2);
-        break;
+    // X is well conditioned after the first iteration; with reduced_slices its
+    // Gram product and the products with the inverses then run with fewer
+    // BF16 slices, the Cholesky factorizations themselves do not.  The
+    // first iteration's correction E is of order 1e-12: 40 bits of it are
+    // more than the result holds.
+    struct ReducedScope {
+      unsigned sites;
+      int slices;
+      ReducedScope(unsigned s_, int n_) : sites(t_tc.reduced_sites), slices(t_tc.reduced_slices) {
+        t_tc.reduced_sites = s_;
+        t_tc.reduced_slices = n_;
       }
-      // ---- Cholesky form: Z_j = X^* X + c_{2j-1} I = R^* R, T_j = X R^{-1} R^{-*}
-      // X is well conditioned here (its singular values lie in [l_s, 1]);
-      // with reduced_slices the Gram and triangular-solve products run with
-      // fewer BF16 slices, the Cholesky factorizations themselves do not
-      struct ReducedScope {
-        unsigned sites;
-        int slices;
-        ReducedScope(int rs) : sites(t_tc.reduced_sites), slices(t_tc.reduced_slices) {
-          if (rs == 5 || rs == 6) {
-            t_tc.reduced_sites = (1u << GS_GRAM) | (1u << GS_TRSM_F_UPD) | (1u << GS_TRSM_F_DIAG) |
-                                 (1u << GS_TRSM_B_UPD) | (1u << GS_TRSM_B_DIAG);
-            t_tc.reduced_slices = rs;
-          }
-        }
-        ~ReducedScope() {
-          t_tc.reduced_sites = sites;
-          t_tc.reduced_slices = slices;
-        }
-      } reduced_scope(reduced_slices);
-      T* G = ar.get<T>(nn * P);
-      T* Z = ar.get<T>(nn * P * r);
-      T* Rinv = ar.get<T>((size_t)NB_CHOL * n * P * r);
-      T* Yt = ar.get<T>(nn * P * r);
-      T* Tt = ar.get<T>(nn * P * r);
-      int* info = ar.get<int>(P * r);
-      GemmArgs<T> g;
-      g.batch = P;
-      g.m = n; g.n = n; g.k = n; g.opA = OP_C; g.opB = OP_N;
-      g.A = X; g.lda = n; g.sA = nn;
-      g.B = X; g.ldb = n; g.sB = nn;
-      g.C = G; g.ldc = n; g.sC = nn;
-      g.alpha = one; g.beta = zer; g.uplo = 1;
-      g.site = GS_GRAM;
-      gemm(g, st);
-      double shifts[R_MAX];
-      for (int j = 0; j < r; ++j) shifts[j] = pl.c[s][2 * j];
-      shift_terms<T>(st, n, G, n, nn, shifts, r, Z, n, nn, P);
-      cholesky<T>(st, n, Z, n, nn, Rinv, (long long)NB_CHOL * n, info, P * r);
-      bool ok = true;
-      if (!sync_free) {
-        d2h(cx, cx.hs.i, info, sizeof(int) * P * r);
-        for (int q = 0; q < P * r; ++q) ok = ok && (cx.hs.i[q] == 0);
+      ~ReducedScope() {
+        t_tc.reduced_sites = sites;
+        t_tc.reduced_slices = slices;
       }
-      if (!ok) {
-        // non-positive pivot: redo this iteration in QR form
-        ar.release(mk2);
-        use_qr = true;
-        if (pd) pd->chol_fallback += 1;
-        continue;
-      }
-      trsm_pair<T>(st, ar, n, X, n, nn, r, Z, n, nn, Rinv, (long long)NB_CHOL * n, Yt, Tt, n, nn, P * r);
-      double aa[R_MAX];
-      for (int j = 0; j < r; ++j) aa[j] = pl.a[s][j];
-      sum_terms<T>(st, n, pl.mhat[s], X, n, nn, aa, r, Tt, n, nn, Xn, n, nn, P);
-      ar.release(mk2);
-      break;
+    };
+    if (s == 0) {
+      ReducedScope scope(1u << GS_ZOLO_POLISH, 5);
+      zolo_first<T>(st, ar, pl, n, P, X, Xn);
+    } else {
+      const bool fewer = reduced_slices == 5 || reduced_slices == 6;
+      ReducedScope scope(fewer ? (1u << GS_GRAM) | (1u << GS_INV_SUM) | (1u << GS_INV_APPLY) : 0u,
+                         fewer ? reduced_slices : 7);
+      zolo_next<T>(st, ar, pl, s, n, P, X, Xn);
     }
-    std::swap(X, Xn);
-    (void)mone;
+    X = Xn;
   }
-  axpby<T>(st, n, n, 1.0, X, n, nn, 0.0, W, n, nn, P);
+  if (X != W) axpby<T>(st, n, n, 1.0, X, n, nn, 0.0, W, n, nn, P);
   ar.release(mk);
 }
 
-template void zolo_pd<double>(Ctx&, Arena&, int, int, const double*, double*, PolarDiag*, int, int, bool);
-template void zolo_pd<z64>(Ctx&, Arena&, int, int, const z64*, z64*, PolarDiag*, int, int, bool);
+template void zolo_pd<double>(Ctx&, Arena&, int, int, const double*, double*, PolarDiag*, int, int);
+template void zolo_pd<z64>(Ctx&, Arena&, int, int, const z64*, z64*, PolarDiag*, int, int);
 
 // ---------------------------------------------------------------- CSD
 template <class T>
@@ -294,7 +393,6 @@ int csd_impl(Ctx& cx, Arena& ar, int n, const T* A1, int lda1, const T* A2, int 
   if (info) {
     info->orth_err[0] = orth[0];
     info->orth_err[1] = orth[1];
-    info->chol_fallback = pd.chol_fallback;
   }
   // Algorithm 2, lines 2-3, for block i: A_i = Q_i R_i, H_i = Q~ R~,
   // W_i = Q_i Q~^* (diag(R) >= 0); H_i is kept
@@ -622,7 +720,6 @@ int polar_impl(Ctx& cx, Arena& ar, int n, const T* A, int lda, T* Wo, int ldw, T
       info->r_terms[s] = s < pl.steps ? pl.r[s] : 0;
       info->ell[s] = s < pl.steps ? pl.ell[s] : 0.0;
     }
-    info->chol_fallback = pd.chol_fallback;
     info->orth_err[0] = orth;
   }
   ZCSD_CUDA(cudaStreamSynchronize(st));
@@ -682,30 +779,30 @@ bool is_device_ptr(const void* p) {
 
 // Upper bound of the workspace (bytes) needed by a call; run_with_ws also
 // grows the arena and retries if a bound turns out short.
-size_t polar_bytes(long long n, int P, size_t es) {
-  const long long nn = n * n;
-  const long long r = R_MAX;
-  long long qr = 2 * (2 * nn) * P * r                                         // M, E
-                 + (long long)ceil_div(n, NB_OUT) * (n + 1 + NB_OUT) * NB_OUT * P * r  // Y
-                 + (long long)ceil_div(n, NB_OUT) * NB_OUT * NB_OUT * P * r           // T
-                 + (long long)(5 * NB_OUT + (MAX_SUM + 1) * NB_QR) * n * P * r;         // W parts, W2
-  long long ch = nn * P + 3 * nn * P * r + (long long)NB_CHOL * n * P * r * (2 + MAX_SUM);
-  return (size_t)((2 * nn * P + std::max(qr, ch)) * es) + 64 * 256;
+size_t polar_bytes(long long n, int P, size_t es, bool tc) {
+  const long long nn = n * n, r = R_MAX;
+  // zolo_first's E, G, F and zolo_next's Z, N per term; the recursion's W, V
+  // (n^2 / 4 each at the top, batch P r) and the iterates
+  const long long words = nn * P * (6 * r + 4);
+  // the slices of the r-term sum, 7 BF16 slices of both operands (complex:
+  // two real terms at a time)
+  const size_t slices = tc ? (size_t)(28 * (n + 128) * (n + 128)) * P * (es == 8 ? r : 2) : 0;
+  return (size_t)(words * es) + slices + 64 * 256;
 }
 
-size_t heig_bytes(long long n, size_t es) {
+size_t heig_bytes(long long n, size_t es, bool tc) {
   const long long nn = n * n;
   long long qr = (long long)ceil_div(n, NB_OUT) * (n + NB_OUT) * NB_OUT +
                  (long long)ceil_div(n, NB_OUT) * NB_OUT * NB_OUT + (long long)(5 * NB_OUT + (MAX_SUM + 1) * NB_QR) * n;
   long long leaves = 5 * std::min<long long>(LEAF_MAX, n) * n + 64 * n;  // packed V, T, S, P and FP32 columns: sum sz^2 <= n leaf
-  return (size_t)((7 * nn + std::max(qr, leaves)) * es) + polar_bytes(n, 1, es) + (size_t)(3 * n + 2048) * 8 + 64 * 256;
+  return (size_t)((7 * nn + std::max(qr, leaves)) * es) + polar_bytes(n, 1, es, tc) + (size_t)(3 * n + 2048) * 8 + 64 * 256;
 }
 
-size_t csd_bytes(long long n, size_t es) {
+size_t csd_bytes(long long n, size_t es, bool tc) {
   const long long nn = n * n;
   size_t fixed = (size_t)(11 * nn * es) + (size_t)(6 * n + 2048) * 8 + 64 * 256;
-  size_t alg2 = (size_t)(7 * nn * es) + polar_bytes(1, 1, es);
-  return fixed + std::max({polar_bytes(n, 2, es), heig_bytes(n, es), alg2 + (size_t)(2 * nn * es)});
+  size_t alg2 = (size_t)(7 * nn * es);
+  return fixed + std::max({polar_bytes(n, 2, es, tc), heig_bytes(n, es, tc), alg2 + (size_t)(2 * nn * es)});
 }
 
 int ensure_ws(Ctx& cx, size_t bytes) {
@@ -850,7 +947,7 @@ template <class T>
 int csd_typed(csd_ctx* ctx, int n, const void* A1, int lda1, const void* A2, int lda2, void* U1, int ldu1, void* U2,
               int ldu2, void* V1, int ldv1, double* theta, int* rank, csd_info* info) {
   Ctx& cx = ctx->cx;
-  const size_t need = csd_bytes(n, sizeof(T)) + (size_t)8 * n * n * sizeof(T);
+  const size_t need = csd_bytes(n, sizeof(T), cx.tensor_cores) + (size_t)8 * n * n * sizeof(T);
   return run_with_ws(cx, need, info, [&](Arena& ar) -> int {
     Mat<T> a1 = view_in<T>(cx, ar, A1, lda1, n, n);
     Mat<T> a2 = view_in<T>(cx, ar, A2, lda2, n, n);
@@ -875,7 +972,7 @@ int csd_typed(csd_ctx* ctx, int n, const void* A1, int lda1, const void* A2, int
 template <class T>
 int polar_typed(csd_ctx* ctx, int n, const void* A, int lda, void* W, int ldw, void* H, int ldh, csd_info* info) {
   Ctx& cx = ctx->cx;
-  const size_t need = polar_bytes(n, 1, sizeof(T)) + (size_t)8 * n * n * sizeof(T);
+  const size_t need = polar_bytes(n, 1, sizeof(T), cx.tensor_cores) + (size_t)8 * n * n * sizeof(T);
   return run_with_ws(cx, need, info, [&](Arena& ar) -> int {
     Mat<T> a = view_in<T>(cx, ar, A, lda, n, n);
     Mat<T> w = view_out<T>(ar, W, ldw, n, n);
@@ -894,7 +991,7 @@ int polar_typed(csd_ctx* ctx, int n, const void* A, int lda, void* W, int ldw, v
 template <class T>
 int heig_typed(csd_ctx* ctx, int n, const void* B, int ldb, double* lam, void* V, int ldv, csd_info* info) {
   Ctx& cx = ctx->cx;
-  const size_t need = heig_bytes(n, sizeof(T)) + (size_t)4 * n * n * sizeof(T);
+  const size_t need = heig_bytes(n, sizeof(T), cx.tensor_cores) + (size_t)4 * n * n * sizeof(T);
   return run_with_ws(cx, need, info, [&](Arena& ar) -> int {
     Mat<T> b = view_in<T>(cx, ar, B, ldb, n, n);
     Mat<T> v = view_out<T>(ar, V, ldv, n, n);
@@ -913,8 +1010,8 @@ template <class T>
 int csd_rect_typed(csd_ctx* ctx, int m1, int m2, int n, const void* A1, int lda1, const void* A2, int lda2, void* U1,
                    int ldu1, void* U2, int ldu2, void* V1, int ldv1, double* theta, int* rank, csd_info* info) {
   Ctx& cx = ctx->cx;
-  const size_t need = csd_bytes(n, sizeof(T)) + (size_t)(4 * (long long)(m1 + m2) * n + 8LL * n * n) * sizeof(T) +
-                      heig_bytes(std::max(m1, m2), sizeof(T)) / 4;
+  const size_t need = csd_bytes(n, sizeof(T), cx.tensor_cores) + (size_t)(4 * (long long)(m1 + m2) * n + 8LL * n * n) * sizeof(T) +
+                      heig_bytes(std::max(m1, m2), sizeof(T), false) / 4;
   return run_with_ws(cx, need, info, [&](Arena& ar) -> int {
     Mat<T> a1 = view_in<T>(cx, ar, A1, lda1, m1, n);
     Mat<T> a2 = view_in<T>(cx, ar, A2, lda2, m2, n);
@@ -941,7 +1038,7 @@ template <class T>
 int complete_v2_typed(csd_ctx* ctx, int n, const void* A3, int lda3, const void* A4, int lda4, const void* U1,
                       int ldu1, const void* U2, int ldu2, const double* theta, void* V2, int ldv2, csd_info* info) {
   Ctx& cx = ctx->cx;
-  const size_t need = heig_bytes(n, sizeof(T)) + (size_t)8 * n * n * sizeof(T);
+  const size_t need = heig_bytes(n, sizeof(T), cx.tensor_cores) + (size_t)8 * n * n * sizeof(T);
   return run_with_ws(cx, need, info, [&](Arena& ar) -> int {
     Mat<T> a3 = view_in<T>(cx, ar, A3, lda3, n, n);
     Mat<T> a4 = view_in<T>(cx, ar, A4, lda4, n, n);

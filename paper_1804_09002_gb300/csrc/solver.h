@@ -18,7 +18,8 @@ struct Plan {
   int steps = 0;
   int r[4];
   double ell[4];
-  double c[4][2 * R_MAX], a[4][R_MAX], mhat[4], sqrtc[4][R_MAX], w[4][R_MAX];
+  double c[4][2 * R_MAX], a[4][R_MAX], mhat[4];
+  double sqrtc[4][R_MAX], w[4][R_MAX];  // sqrt(c_{2j-1}), mhat a_j / sqrt(c_{2j-1})
 };
 
 struct Ctx {
@@ -53,7 +54,6 @@ enum TestFlags : unsigned {
 };
 
 struct PolarDiag {
-  int chol_fallback = 0;
   int iters = 0;  // Zolo-pd iterations run
 };
 
@@ -70,14 +70,13 @@ void d2h(Ctx& cx, void* dst, const void* src, size_t bytes);
 // W_p = polar factor of X0_p for p < P (Zolo-pd, Section 5); X0 and W are
 // P consecutive n x n matrices (ld n).  Workspace comes from `ar`.
 // stop_after > 0 stops after that many iterations (the iterate X_k).
-// reduced_slices = 5 or 6 runs the Gram and triangular-solve products of the
-// Cholesky-form iterations with that many BF16 slices (tensor-core path).
-// sync_free: no device-to-host read (the Cholesky pivot check is skipped:
-// a non-positive pivot leaves NaN, which the caller's checks catch), so the
-// call can be captured in a CUDA graph.
+// reduced_slices = 5 or 6 runs the Gram product and the products with the
+// inverses of the Cholesky-form iterations with that many BF16 slices
+// (tensor-core path).  No device-to-host read, so the call can be captured in
+// a CUDA graph.
 template <class T>
 void zolo_pd(Ctx& cx, Arena& ar, int n, int P, const T* X0, T* W, PolarDiag* pd, int stop_after = 0,
-             int reduced_slices = 0, bool sync_free = false);
+             int reduced_slices = 0);
 
 // Counters of one Zolo-eig call.
 struct EigDiag {

@@ -693,6 +693,11 @@ bool tc_will_handle(const GemmArgs<double>& g) {
   // FP64 pipe is ~20x slower than the sliced tensor-core rate, so products
   // with k >= 512 (the W = Y^* C panels of the blocked QR) also go there.
   if (!(t_tc.enabled && t_tc.ar && ((t_tc.sites >> g.site) & 1u) && tc_gemm_supported(g))) return false;
+  // Below about 24 M multiply-adds the FP64 pipe is done (80 us, spread over
+  // all SMs by small tiles) before the slicing and its launches pay.
+  const double work = (double)g.m * g.n * g.k * g.batch * std::max(1, g.nsum) *
+                      (g.uplo ? 0.5 : 1.0) * (g.kflags ? 0.5 : 1.0);
+  if (work < 24e6) return false;
   if (g.m >= TC_BM && g.n >= TC_BN && g.k >= 64) return true;
   return g.m >= 32 && g.n >= 32 && g.k >= 512;
 }
@@ -808,6 +813,8 @@ bool tc_will_handle_complex(const GemmArgs<z64>& g) {
   if (g.nsum != 1 || g.kbal || g.alpha.y != 0.0 || g.beta.y != 0.0) return false;
   GemmArgs<double> r;
   r.m = g.m; r.n = g.n; r.k = g.k; r.site = g.site; r.ksplit = std::max(1, g.ksplit);
+  r.batch = g.batch; r.uplo = g.uplo; r.kflags = g.kflags;
+  r.nsum = 4;  // its work in real multiply-adds
   return tc_will_handle(r);
 }
 
