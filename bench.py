@@ -44,11 +44,11 @@ def parse():
     ap.add_argument("--sample-n", type=int, default=1024,
                     help="oracle sample size for the CPU baseline (about 20 s on 16 Grace cores)")
     ap.add_argument("--tc", type=int, default=1,
-                    help="1 (default): real FP64 products on the tcgen05 tensor cores (exact BF16 slicing); 0: FP64 pipe")
+                    help="1 (default): real FP64 products on the tcgen05 tensor cores (exact BF16 residue products); 0: FP64 pipe")
     ap.add_argument("--compare-fp64", type=int, default=1,
                     help="with --tc 1, also time the FP64-pipe path (same workload, same accuracy checks)")
     ap.add_argument("--mixed-slices", type=int, default=6,
-                    help="also time the mixed-precision path: Cholesky-iteration products with 5 or 6 BF16 slices "
+                    help="also time the mixed-precision path: Cholesky-iteration products with fewer bits (5: 45, 6: 51) "
                          "(0 = skip)")
     ap.add_argument("--mixed-scope", type=int, default=1,
                     help="bit 0: the two polar decompositions, bit 1: Zolo-eig's polar decompositions")
@@ -321,11 +321,14 @@ def accuracy(R, A1, A2, th_known, n, dev):
             "orth_2norm_over_u": orth2 / U, "rank": rk, "bar_over_u": 50 * n}
 
 
+# BF16 products per FP64-equivalent product of up to 4096 terms (tc_gemm.cu).
+RNS_PRODUCTS = 14
+
 # DRAM traffic of the tensor-core product kernel per launch, from one ncu
 # capture (dram__bytes_read.sum + dram__bytes_write.sum over every launch of
 # the kernel in one step), with the hash of the kernel source it was taken
 # at; reported only while tc_gemm.cu is unchanged since the capture.
-TRAFFIC = {"tc_gemm": {"bytes_per_launch": 289092468, "src_hash": "60e10541738decac",
+TRAFFIC = {"tc_gemm": {"bytes_per_launch": 405789471, "src_hash": "06f22e33f665ba08",
                       "profile": "profiles/tc_gemm_kernel_csd_n4096_traffic.md"}}
 
 
@@ -382,8 +385,8 @@ def run_gemm(args):
         fl = 2.0 * n ** 3
         res["tensor_cores" if engine else "fp64_pipe"] = {
             "ms": ms, "fp64_equivalent_tflops": fl / ms / 1e9,
-            **({"bf16_slice_tflops": 28 * fl / ms / 1e9,
-                "frac_of_bf16_sustained": 28 * fl / ms / 1e9 / peaks().get("bf16_tflops_sustained", 1719.1)}
+            **({"bf16_residue_tflops": RNS_PRODUCTS * fl / ms / 1e9,
+                "frac_of_bf16_sustained": RNS_PRODUCTS * fl / ms / 1e9 / peaks().get("bf16_tflops_sustained", 1719.1)}
                if engine else {"frac_of_fp64_unit_peak": fl / ms / 1e9 / fp64_alu_peak_tflops()})}
     err = float(torch.max(torch.abs(C - A @ Bm)))
     ctx.close()
@@ -547,7 +550,7 @@ def main():
                  "slices": args.mixed_slices, "scope": args.mixed_scope,
                  "accuracy": accuracy(Rx, A1, A2, th_known, n, dev), "clocks": ckx,
                  "what": "Gram and triangular-solve products of the Cholesky-form Zolo-pd iteration with "
-                         f"{args.mixed_slices} BF16 slices; everything else FP64-accurate (7 slices)"}
+                         f"{45 if args.mixed_slices == 5 else 51} bits; everything else FP64-accurate (56)"}
         ctx.set_mixed_precision(7, 0)
     # ---- e2e: same call with pinned host buffers (copies inside the call)
     e2e = None
@@ -576,25 +579,26 @@ def main():
     flops_per_launch = prof.flops[dom] / max(prof.count[dom], 1)
     pk = peaks()
     if kinds[dom] == "tc_gemm":
-        # 28 BF16 slice products per FP64-equivalent product, against the
-        # measured dense BF16 peak (slicing included in the kernel time)
+        # 14 BF16 residue products per FP64-equivalent product (15 for sums of
+        # more than 4096 terms, fewer where fewer bits are kept), against the
+        # measured dense BF16 peak (conversions included in the kernel time)
         peak = pk.get("bf16_tflops_sustained", 1719.1)
         fp64eq = flops_per_launch / (avg_ms / 1e3) / 1e12 if avg_ms > 0 else 0.0
-        achieved = 28.0 * fp64eq
+        achieved = RNS_PRODUCTS * fp64eq
         tr, tr_src = traffic_for("tc_gemm")
         roof = {"kernel": "tc_gemm", "bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": tr, "traffic_source": tr_src,
                 "peak_source": "MEASURED_PEAKS.json bf16_tflops_sustained (of measured)",
                 "launches_per_step": prof.count[dom], "avg_launch_ms": avg_ms,
                 "fp64_equivalent_tflops": fp64eq, "method_frac_of_bf16_peak": fp64eq / peak,
-                "work_per_launch": "28 x 2mnk BF16 slice flops (2mnk FP64-equivalent) over the tiles executed"}
+                "work_per_launch": "14 x 2mnk BF16 residue flops (2mnk FP64-equivalent) over the tiles executed"}
     else:
         peak = fp64_alu_peak_tflops()
         achieved = flops_per_launch / (avg_ms / 1e3) / 1e12 if avg_ms > 0 else 0.0
         roof = {"kernel": kinds[dom], "bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": None,
                 "peak_source": "FP64 FMA pipe: 152 SMs x 2 DFMA/clk x 2 flop x 2070 MHz"}
-    products = ("tcgen05 tensor cores, exact BF16 slicing (FP64-accurate), FP64 pipe for the rest" if args.tc
+    products = ("tcgen05 tensor cores, exact BF16 residue products (FP64-accurate), FP64 pipe for the rest" if args.tc
                 and not cfg["cplx"] else "FP64 FMA pipe")
     metric = f"s/CSD at n={n} ({'complex128' if cfg['cplx'] else 'FP64'})"
     line = {

@@ -223,14 +223,13 @@ int csd_profile_enable(csd_ctx* ctx, int enable);
  * product on the FP64 pipe; otherwise bit s of `enable` selects the products
  * of call site s (the site numbering of csd_profile); enable = -1 selects
  * every site.
- * The products stay FP64-accurate: each operand is split exactly into seven
- * BF16 slices with per-row / per-column power-of-two scaling, the slice
- * products are accumulated exactly (FP32 over 128 k, then a 64-bit integer)
- * except the smallest ones (error of the same order as an FP64 product).
- * The rows below X in the trailing update of the stacked [X; sqrt(c) I]
- * factorization (site 3) are of the size of sqrt(c) and need accuracy
- * relative to themselves: that product is also balanced along its inner
+ * The products stay FP64-accurate: each operand is rounded to 56-bit integers
+ * with per-row / per-column power-of-two scaling, and the integer product is
+ * assembled from exact products modulo 14 (long sums: 15) small moduli.  The
+ * trailing update of the blocked QR (site 3) is also balanced along its inner
  * dimension by powers of two (A D, D^-1 B, D = diag of the row maxima of B).
+ * Small products, where the conversion would cost more than it saves, stay on
+ * the FP64 pipe.
  * Complex products with real alpha and beta run as two real grouped sums
  * over the interleaved parts (Re C = Re A Re B - Im A Im B,
  * Im C = Re A Im B + Im A Re B); grouped complex sums and the balanced
@@ -239,24 +238,22 @@ int csd_set_tensor_cores(csd_ctx* ctx, int enable);
 int csd_profile_read(csd_ctx* ctx, csd_profile* out);
 
 /* Leaf size of Zolo-eig's spectral divide and conquer (Section 5): blocks of
- * at most `leaf` rows (1..1024, default 256) are not split further but
- * diagonalised by two-sided cyclic Jacobi (parallel tournament order), all
- * leaves of a call batched into the same launches, one CTA per column pair
- * and round; when every leaf has at most 64 rows, one CTA per leaf runs the
- * whole iteration in shared memory.  The paper leaves the recursion's
- * stopping size open.
+ * at most `leaf` rows (1..1024, default 1024) are not split further but
+ * diagonalised directly, all leaves of a call in the same launches: FP32
+ * Jacobi for a starting basis, FP64 refinement, FP64 Jacobi for what that
+ * leaves open.  The paper leaves the recursion's stopping size open.
  * Returns 0, -1 (NULL context) or -2 (out of range). */
 int csd_set_eig_leaf(csd_ctx* ctx, int leaf);
 
 /* Mixed precision on the tensor-core path (csd_set_tensor_cores): once the
- * first, QR-form iteration has mapped the singular values into
+ * first iteration has mapped the singular values into
  * [l_1, 1] = [0.4565, 1], the Cholesky-form iteration works on a well
- * conditioned X, and its Gram product X^* X and the products of its paired
- * triangular solves may run with `slices` = 5 or 6 BF16 slices per operand
- * (40 or 48 bits, 15 or 21 slice products instead of 28) while the QR
- * iteration, the Cholesky factorizations, H_i, B, Zolo-eig's subspace
- * products and the assembly keep 7 (FP64-accurate).  scope bit 0: the two
- * polar decompositions of csd_polar (and polar()); bit 1: the polar
+ * conditioned X, and its Gram product X^* X and the products with the inverses
+ * may keep 45 (`slices` = 5) or 51 (6) bits of their operands (12 or 13
+ * modular products instead of 14) while the first iteration, the Cholesky
+ * factorizations, H_i, B, Zolo-eig's subspace products and the assembly keep
+ * 56 (FP64-accurate).  scope bit 0: the two polar decompositions of csd_polar
+ * (and polar()); bit 1: the polar
  * decompositions inside Zolo-eig.  slices = 7 or scope = 0 is the default
  * FP64-accurate path.  The result is checked like any other: angles,
  * backward error and orthogonality against the 50 n u bar.
@@ -334,9 +331,8 @@ int csd_set_zolo_control(csd_ctx* ctx, int max_extra_passes, int stop_after);
  *     copy or MMA; the wait runs out, the launch writes NaN outputs, sets
  *     the device error flag and the call returns CSD_ERR_DEVICE_TIMEOUT.
  *     The context stays usable.
- *   tc_flush_every > 0: the tensor-core kernel writes its 64-bit integer
- *     partial sum out to C every this many 128-k drains (default: every
- *     120 drains, i.e. only for K > 15 360).
+ *   tc_flush_every: accepted and without effect (the partial sums of long
+ *     products need no write-out).
  * Returns 0, -1 (NULL context), -2 (unknown flag), -3 / -4 (negative). */
 #define CSD_TEST_REJECT_EIG_SPLITS 1u
 int csd_set_test_hooks(csd_ctx* ctx, unsigned flags, long long tc_probe_wait, int tc_flush_every);

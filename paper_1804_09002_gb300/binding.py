@@ -262,7 +262,7 @@ class Context:
             lib.csd_set_stream(self._h, None)
 
     def set_tensor_cores(self, enable=True, sites=-1):
-        """Run real FP64 products on the tcgen05 tensor cores (sliced BF16,
+        """Run real FP64 products on the tcgen05 tensor cores (modular BF16,
         FP64-accurate) instead of the FP64 FMA pipe; `sites` is a bit mask
         over the GEMM call sites (csd_profile.SITES), -1 = all."""
         st = lib.csd_set_tensor_cores(self._h, (sites if sites else 0) if enable else 0)
@@ -287,8 +287,8 @@ class Context:
             raise CSDError(st, "csd_set_eig_leaf")
 
     def set_mixed_precision(self, slices=6, scope=1):
-        """Cholesky-iteration products of Zolo-pd with 5 or 6 BF16 slices
-        (scope bit 0: the CSD's polars, bit 1: Zolo-eig's); 7 = off."""
+        """Cholesky-iteration products of Zolo-pd with 45 (slices = 5) or 51
+        (6) bits (scope bit 0: the CSD's polars, bit 1: Zolo-eig's); 7 = off."""
         st = lib.csd_set_mixed_precision(self._h, int(slices), int(scope))
         if st != 0:
             raise CSDError(st, "csd_set_mixed_precision")

@@ -29,22 +29,18 @@ static int pick_ksplit(int m, int n, int k, int batch, int bm, int kmin = 256) {
   return best;
 }
 
-// Split-K factor of a product: the FP64-pipe choice `ks`, or, when the
-// tensor-core path takes the product, its own choice (one CTA per SM there);
-// both at most `cap`, the partial buffers the caller holds.
+// Split-K factor of a product: the FP64-pipe choice `ks`, at most `cap`, the
+// partial buffers the caller holds, or 1 when the tensor-core path takes the
+// product (its items, one per modulus, fill the SMs).
 template <class T>
 static int resolve_ksplit(GemmArgs<T>& g, int ks, int cap) {
   g.ksplit = std::max(1, std::min(ks, cap));
   GemmArgs<T> probe = g;
   probe.ksplit = 1;
   if constexpr (std::is_same<T, double>::value) {
-    if (tc_will_handle(probe)) g.ksplit = tc_pick_ksplit(probe, cap);
+    if (tc_will_handle(probe)) g.ksplit = 1;
   } else {
-    if (tc_will_handle_complex(probe)) {
-      GemmArgs<double> r;  // the real products it becomes: same tiles
-      r.m = g.m; r.n = g.n; r.k = g.k; r.batch = g.batch;
-      g.ksplit = tc_pick_ksplit(r, cap);
-    }
+    if (tc_will_handle_complex(probe)) g.ksplit = 1;
   }
   return g.ksplit;
 }

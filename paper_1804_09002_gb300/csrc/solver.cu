@@ -283,29 +283,29 @@ void zolo_pd(Ctx& cx, Arena& ar, int n, int P, const T* X0, T* W, PolarDiag* pd,
     T* Xn = s + 1 == steps && X != W && X0 != W ? W : (X == Xa ? Xb : Xa);
     if (pd) pd->iters += 1;
     // X is well conditioned after the first iteration; with reduced_slices its
-    // Gram product and the products with the inverses then run with fewer
-    // BF16 slices, the Cholesky factorizations themselves do not.  The
-    // first iteration's correction E is of order 1e-12: 40 bits of it are
-    // more than the result holds.
+    // Gram product and the products with the inverses then keep fewer bits of
+    // their operands, the Cholesky factorizations themselves do not.  The
+    // first iteration's correction E is of order 1e-12 or less: 24 bits of it
+    // reach 1e-19.
     struct ReducedScope {
       unsigned sites;
-      int slices;
-      ReducedScope(unsigned s_, int n_) : sites(t_tc.reduced_sites), slices(t_tc.reduced_slices) {
+      int bits;
+      ReducedScope(unsigned s_, int n_) : sites(t_tc.reduced_sites), bits(t_tc.reduced_bits) {
         t_tc.reduced_sites = s_;
-        t_tc.reduced_slices = n_;
+        t_tc.reduced_bits = n_;
       }
       ~ReducedScope() {
         t_tc.reduced_sites = sites;
-        t_tc.reduced_slices = slices;
+        t_tc.reduced_bits = bits;
       }
     };
     if (s == 0) {
-      ReducedScope scope(1u << GS_ZOLO_POLISH, 5);
+      ReducedScope scope(1u << GS_ZOLO_POLISH, 24);
       zolo_first<T>(st, ar, pl, n, P, X, Xn);
     } else {
       const bool fewer = reduced_slices == 5 || reduced_slices == 6;
       ReducedScope scope(fewer ? (1u << GS_GRAM) | (1u << GS_INV_SUM) | (1u << GS_INV_APPLY) : 0u,
-                         fewer ? reduced_slices : 7);
+                         fewer ? (reduced_slices == 5 ? 45 : 51) : 56);
       zolo_next<T>(st, ar, pl, s, n, P, X, Xn);
     }
     X = Xn;
@@ -784,9 +784,8 @@ size_t polar_bytes(long long n, int P, size_t es, bool tc) {
   // zolo_first's E, G, F and zolo_next's Z, N per term; the recursion's W, V
   // (n^2 / 4 each at the top, batch P r) and the iterates
   const long long words = nn * P * (6 * r + 4);
-  // the slices of the r-term sum, 7 BF16 slices of both operands (complex:
-  // two real terms at a time)
-  const size_t slices = tc ? (size_t)(28 * (n + 128) * (n + 128)) * P * (es == 8 ? r : 2) : 0;
+  // residues of the r-term sum on the tensor cores (complex: two real terms)
+  const size_t slices = tc ? tc_gemm_bytes(n, n, n, es == 8 ? (int)r : 2) * P : 0;
   return (size_t)(words * es) + slices + 64 * 256;
 }
 
@@ -856,7 +855,6 @@ int run_with_ws(Ctx& cx, size_t need, csd_info* info, F body) {
       t_tc.ar = &ar;
       t_tc.err = tc_err;
       t_tc.probe_wait = cx.tc_probe_wait;
-      t_tc.flush_every = cx.tc_flush_every;
       status = body(ar);
       if (tc_err) {
         int h = 0;
@@ -1084,7 +1082,7 @@ int backward_typed(csd_ctx* ctx, int n, const void* U1, int ldu1, const void* U2
 int gemm_typed(csd_ctx* ctx, int opA, int opB, int m, int n, int k, double alpha, const double* A, int lda,
                const double* B, int ldb, double beta, double* C, int ldc, int engine) {
   Ctx& cx = ctx->cx;
-  const size_t need = (size_t)16 * ((size_t)(m + 128) * (k + 64) + (size_t)(n + 128) * (k + 64)) + (1 << 20);
+  const size_t need = tc_gemm_bytes(m, n, std::max(k, 1), 1) + (1 << 20);
   cx.force_tc_err = engine == 1;
   const int st = run_with_ws(cx, need, nullptr, [&](Arena& ar) -> int {
     GemmArgs<double> g;

@@ -39,7 +39,7 @@ struct Ctx {
   int zolo_stop_after = 0;    // polar(): > 0 returns the iterate X_k after k iterations (k <= plan steps)
   unsigned test_flags = 0;    // TEST_* below (fault injection on the host; default off)
   long long tc_probe_wait = 0;  // tensor-core kernel: polls of a barrier nothing signals (0 = none)
-  int tc_flush_every = 0;       // tensor-core kernel: drains between int64 write-outs (0 = default)
+  int tc_flush_every = 0;       // accepted and without effect (csd_set_test_hooks)
   bool force_tc_err = false;    // the running call needs the tensor-core error flag (csd_gemm)
   int sign_mode = 0;            // 1: canonical column signs of U1, U2, V1 (csd_set_sign_convention)
   double alg2_svd_factor = 1e3;  // SVD polar fallback when ||R~ - R|| / ||R|| > factor n u (< 0: never)
@@ -71,7 +71,7 @@ void d2h(Ctx& cx, void* dst, const void* src, size_t bytes);
 // P consecutive n x n matrices (ld n).  Workspace comes from `ar`.
 // stop_after > 0 stops after that many iterations (the iterate X_k).
 // reduced_slices = 5 or 6 runs the Gram product and the products with the
-// inverses of the Cholesky-form iterations with that many BF16 slices
+// inverses of the Cholesky-form iterations with 45 or 51 bits of the operands
 // (tensor-core path).  No device-to-host read, so the call can be captured in
 // a CUDA graph.
 template <class T>
