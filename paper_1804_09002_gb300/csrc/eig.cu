@@ -3,18 +3,19 @@
 //
 // A split of block B_sub (sz x sz) at the shift s: W = polar((B_sub - sI) /
 // ||B_sub - sI||_F) by Zolo-pd, P = (W + I)/2 projects onto the eigenvectors
-// above s, k = trace(P) of them; [Q1 Q2] = qr(P Omega) with Omega Gaussian
-// gives Q1 spanning range(P), and Q^* B_sub Q is block diagonal up to
+// above s, k = trace(P) of them; [Q1 Q2] = orth([P Omega_1, (I - P) Omega_2])
+// with Omega Gaussian gives Q1 spanning range(P), and Q^* B_sub Q is block
+// diagonal up to
 // ||B'_21||_F, which is the backward error of the split.
 //
 // The recursion runs level by level.  Every block of a level that still
 // needs a split goes through the same launches: the blocks form groups
 // (chosen by a cost model), each block is padded to the group's largest
 // size nb with an identity block, X_p = diag((B_p - s_p I) / ||B_p - s_p I||_F, I), and one
-// batched Zolo-pd, one batched QR and batched products serve the whole
-// group.  The padding is exactly decoupled: polar(diag(X, I)) = diag(polar(X),
-// I); with P padded by zeros, P Omega has zero rows below sz_p, so every
-// Householder reflector is zero there and Q = diag(Q_p, I) exactly.  The
+// batched Zolo-pd, one batched orthonormalisation and batched products serve
+// the whole group.  The padding is exactly decoupled: polar(diag(X, I)) =
+// diag(polar(X), I), and the two bases are padded by the identity, so
+// Q = diag(Q_p, I) exactly.  The
 // host reads the per-block scalars (norms, medians, traces, off-block
 // norms) once per level and attempt, not once per block.
 #include <algorithm>
@@ -158,6 +159,24 @@ __global__ void blk_proj_pad(const T* W, int nb, const int* sz, T* Pm) {
       if (i == j) v = add(v, from_re<T>(0.5));
     }
     Pp[e] = v;
+  }
+}
+
+// Y_p: columns below k_p from W = P Omega, the others from Omega - W = (I - P)
+// Omega, on the leading sz_p x sz_p block; the identity elsewhere, and for a
+// problem without a valid k
+template <class T>
+__global__ void blk_two_bases(const T* W, const T* Om, int nb, const int* sz, const int* k, T* Y) {
+  const int p = blockIdx.y, m = k[p] < 0 ? 0 : sz[p], kp = k[p];
+  const long long nn = (long long)nb * nb;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < nn; e += (long long)gridDim.x * blockDim.x) {
+    const int i = (int)(e % nb), j = (int)(e / nb);
+    T v = from_re<T>(i == j ? 1.0 : 0.0);
+    if (i < m && j < m) {
+      v = W[p * nn + e];
+      if (j >= kp) v = sub(Om[p * nn + e], v);
+    }
+    Y[p * nn + e] = v;
   }
 }
 
@@ -441,12 +460,17 @@ void heig_impl(Ctx& cx, Arena& ar, int n, const T* Bin, int ldb, double* lam, T*
           ar.release(mg);
           continue;
         }
-        // ---- [Q1 Q2] = qr(P Omega), Q1 spans range(P) (Q = diag(Q_p, I)).
-        // With a square Gaussian Omega the leading k columns of P Omega have
-        // a condition number of order k, and so does the error of Q1; a block
-        // whose split fails the off-block test gets one step of subspace
-        // iteration, Q <- qr(P Q), whose leading columns P Q1 ~ Q1 are well
-        // conditioned, before a new shift (and a new polar factor) is tried.
+        // ---- Q1 spans range(P), Q2 its complement (Q = diag(Q_p, I)): the
+        // leading k columns of P Omega and the others of (I - P) Omega, together
+        // orthonormalised by their inverse Cholesky factor.  The two sets are
+        // orthogonal to rounding, so the factor only has their own condition
+        // numbers, of order k^2; two steps of Q <- Q - Q E / 2, E = Q^* Q - I of
+        // order k^2 u, restore orthonormality.  (Householder QR of P Omega took a
+        // fifth of a split, a chain of n / 32 panels.)  Q1 inherits an error of
+        // order k u from the condition of P Omega; a block whose split fails
+        // the off-block test gets one step of subspace iteration from Q, whose
+        // P Q1 ~ Q1 are well conditioned, before a new shift (and a new polar
+        // factor) is tried.
         T* Pm = ar.get<T>(nbb * Pa);
         blk_proj_pad<T><<<dim3(ew_grid(nbb), Pa), 256, 0, st>>>(Wm, nb, dsz, Pm);
         ZCSD_LAUNCH();
@@ -466,14 +490,50 @@ void heig_impl(Ctx& cx, Arena& ar, int n, const T* Bin, int ldb, double* lam, T*
         std::vector<int> cand;  // blocks with a valid k still to be tested
         for (int a = 0; a < Pa; ++a)
           if (k[a] >= 0) cand.push_back(a);
+        const int* dk = upload(ar, st, k);
+        T* Nf = ar.get<T>(nbb * Pa);
         for (int pass = 0; pass < 2 && !cand.empty(); ++pass) {
-          bgemm(OP_N, Pm, pass == 0 ? Om : Qf, Wm);  // P Omega, then P Q
+          T* basis = pass == 0 ? Om : Qf;
+          bgemm(OP_N, Pm, basis, Wm);  // P Omega, then P Q
+          blk_two_bases<T><<<dim3(ew_grid(nbb), Pa), 256, 0, st>>>(Wm, basis, nb, dsz, dk, Tm);
+          ZCSD_LAUNCH();
+          auto gram = [&](const T* A) {  // Wm = A^* A (upper triangle)
+            GemmArgs<T> g;
+            g.batch = Pa;
+            g.m = nb; g.n = nb; g.k = nb; g.opA = OP_C; g.opB = OP_N; g.uplo = 1;
+            g.A = A; g.lda = nb; g.sA = nbb;
+            g.B = A; g.ldb = nb; g.sB = nbb;
+            g.C = Wm; g.ldc = nb; g.sC = nbb;
+            g.alpha = one; g.beta = zer; g.site = GS_EIG;
+            gemm(g, st);
+          };
+          gram(Tm);
+          ZCSD_CUDA(cudaMemsetAsync(Nf, 0, sizeof(T) * nbb * Pa, st));
+          chol_inverse<T>(st, ar, nb, Wm, nb, nbb, Nf, nb, nbb, Pa);
           {
-            const size_t mq = ar.mark();
-            QRStore<T> q = qr_alloc<T>(ar, nb, nb, nb, Pa);
-            qr_factor<T>(st, ar, q, Wm, nb, nbb);
-            qr_form_q<T>(st, ar, q, Qf, nb, nbb);
-            ar.release(mq);
+            GemmArgs<T> g;  // Q = Y N
+            g.batch = Pa;
+            g.m = nb; g.n = nb; g.k = nb; g.opA = OP_N; g.opB = OP_N; g.kflags = K_TO_COL;
+            g.A = Tm; g.lda = nb; g.sA = nbb;
+            g.B = Nf; g.ldb = nb; g.sB = nbb;
+            g.C = Qf; g.ldc = nb; g.sC = nbb;
+            g.alpha = one; g.beta = zer; g.site = GS_EIG;
+            gemm(g, st);
+          }
+          for (int it = 0; it < 2; ++it) {  // Q <- Q - Q E / 2
+            T* from = it == 0 ? Qf : Tm;
+            gram(from);
+            minus_eye<T>(st, nb, Wm, nb, nbb, Nf, nb, nbb, Pa);
+            ReducedScope scope(1u << GS_ZOLO_POLISH, it == 0 ? 45 : 24);
+            GemmArgs<T> g;
+            g.batch = Pa;
+            g.m = nb; g.n = nb; g.k = nb; g.opA = OP_N; g.opB = OP_N;
+            g.A = from; g.lda = nb; g.sA = nbb;
+            g.B = Nf; g.ldb = nb; g.sB = nbb;
+            g.Cin = from; g.ldcin = nb; g.sCin = nbb;
+            g.C = it == 0 ? Tm : Qf; g.ldc = nb; g.sC = nbb;
+            g.alpha = from_re<T>(-0.5); g.beta = one; g.site = GS_ZOLO_POLISH;
+            gemm(g, st);
           }
           // ---- B' = Q^* B_sub Q = ||B_sub - sI||_F Q^* X Q + s I: the shift
           // is added back exactly, so the departure of Q from orthogonality

@@ -103,21 +103,26 @@ void d2h(Ctx& cx, void* dst, const void* src, size_t bytes) {
 // I)^{-1} = Q1 Q2^* / sqrt(c); any basis gives the same term, so the QR factor
 // of Section 5 is not needed).  The shifts c_j are about 4700 apart, which a
 // chain of Cholesky factorizations uses:
-//   * the largest, 8.5e-4: X^* X + c I has condition number 1200; with N its
-//     inverse Cholesky factor, Q1 = X N and Q2 = sqrt(c) N;
-//   * the basis of term j + 1 preconditions term j: the columns of
-//     [Q1; sqrt(rho) Q2], rho = c_j / c_{j+1}, span [X; sqrt(c_j) I], and their
-//     Gram matrix rho I + (1 - rho) Q1^* Q1 has condition number 1 / rho; its
+//   * the two largest, 8.5e-4 and 1.8e-7: with N the inverse Cholesky factor
+//     of X^* X + c I, Q1 = X N and Q2 = sqrt(c) N;
+//   * the basis of term j preconditions the terms below it: the columns of
+//     [Q1; sqrt(rho) Q2], rho = c_i / c_j, span [X; sqrt(c_i) I], and their Gram
+//     matrix rho I + (1 - rho) Q1^* Q1 has condition number 1 / rho; its
 //     inverse Cholesky factor orthonormalises them.  It is positive definite
 //     for every X, so there is no pivot to check.
-// Each step leaves a departure E = Q1^* Q1 + Q2^* Q2 - I of order u / rho,
-// which does not grow along the chain; to first order the term of the exact
-// basis is (Q1 - Q1 E) Q2^*, one more product.  The result is as accurate as
-// with Householder factorizations of the stacked matrices (backward error 14 u
-// against 13 u, at any sigma_min) and all but the 64-column blocks are
+// Two terms follow from each basis, 1 / rho = 4.7e3 and 2.2e7, so that the
+// chain is four factorizations of two problems long (eight of one leave more
+// SMs idle: the factorization of n = 1024 is a chain of 16 blocks of 77 us).
+// Each step leaves a departure E = Q1^* Q1 + Q2^* Q2 - I of order u / rho, 1e-8
+// at most, which does not grow along the chain; the term of the exact basis is
+// Q1 (I + E)^{-1} Q2^*, two more products up to E^3.  The result is as accurate
+// as with Householder factorizations of the stacked matrices (backward error
+// 13 u with either, at any sigma_min) and all but the innermost blocks are
 // products with large K: the Householder panels took a fifth of a
 // decomposition and their updates, with K = 128, most of the rest (polar of
-// n = 2048 130 -> 86 ms, a complex n = 512 decomposition 155 -> 113 ms).
+// n = 2048 130 -> 86 ms, a complex n = 512 decomposition 155 -> 113 ms, with
+// one term per step; two: 62 -> 44 and 82 -> 50 ms, together with the bases of
+// Zolo-eig).
 template <class T>
 static void zolo_first(cudaStream_t st, Arena& ar, const Plan& pl, int n, int P, const T* X, T* Xn) {
   const int r = pl.r[0];
@@ -127,9 +132,10 @@ static void zolo_first(cudaStream_t st, Arena& ar, const Plan& pl, int n, int P,
   const size_t mk = ar.mark();
   T* E = ar.get<T>(sM * P * r);   // Q2 as N, the accumulated inverse factors: scaled by sqrt(c_j) at the end
   T* G = ar.get<T>(nn * P * r);   // Gram matrices Q1^* Q1
-  T* Z = ar.get<T>(nn * P);
-  T* N = ar.get<T>(nn * P);
-  ZCSD_CUDA(cudaMemsetAsync(N, 0, sizeof(T) * nn * P, st));
+  T* F = ar.get<T>(nn * P * r);
+  T* Z = ar.get<T>(2 * nn * P);
+  T* N = ar.get<T>(2 * nn * P);
+  ZCSD_CUDA(cudaMemsetAsync(N, 0, 2 * sizeof(T) * nn * P, st));
   auto gram = [&](const T* A, int lda, long long sA, T* C, long long sC) {
     GemmArgs<T> g;
     g.batch = P;
@@ -143,35 +149,41 @@ static void zolo_first(cudaStream_t st, Arena& ar, const Plan& pl, int n, int P,
   // rows of [Q1; Q2] times N: together while a launch costs more than the
   // zeros of Q2, apart above
   const bool together = n <= 256;
-  for (int j = r - 1; j >= 0; --j) {
-    T* Ej = E + j * sM;
-    const bool first = j == r - 1;
-    const double c = pl.c[0][2 * j], rho = first ? 1.0 : c / pl.c[0][2 * (j + 1)];
-    if (first) {
-      gram(X, n, nn, G + j * nn, nn * r);
-      scale_shift<T>(st, n, 1.0, G + j * nn, n, nn * r, c, Z, n, nn, P);
-    } else {
-      scale_shift<T>(st, n, 1.0 - rho, G + (j + 1) * nn, n, nn * r, rho, Z, n, nn, P);
+  T* GX = F;  // X^* X
+  gram(X, n, nn, GX, nn);
+  for (int base = r; base > 0;) {  // terms base - 1 and base - 2 from term base (base == r: from X itself)
+    const int cnt = std::min(2, base);
+    const bool first = base == r;
+    for (int i = 0; i < cnt; ++i) {
+      const double c = pl.c[0][2 * (base - 1 - i)];
+      const double rho = first ? 0.0 : c / pl.c[0][2 * base];
+      if (first) scale_shift<T>(st, n, 1.0, GX, n, nn, c, Z + i * nn * P, n, nn, P);
+      else scale_shift<T>(st, n, 1.0 - rho, G + base * nn, n, nn * r, rho, Z + i * nn * P, n, nn, P);
     }
-    chol_inverse<T>(st, ar, n, Z, n, nn, N, n, nn, P);
-    GemmArgs<T> g;
-    g.batch = P;
-    g.m = (!first && together) ? m2 : n; g.n = n; g.k = n; g.opA = OP_N; g.opB = OP_N; g.kflags = K_TO_COL;
-    if (first) { g.A = X; g.lda = n; g.sA = nn; }
-    else { g.A = Ej + sM; g.lda = m2; g.sA = sM * r; }
-    g.B = N; g.ldb = n; g.sB = nn;
-    g.C = Ej; g.ldc = m2; g.sC = sM * r;
-    g.alpha = one; g.beta = zer; g.site = GS_ZOLO_Q;
-    gemm(g, st);
-    if (first) {
-      axpby<T>(st, n, n, 1.0, N, n, nn, 0.0, Ej + n, m2, sM * r, P);
-    } else if (!together) {
-      g.A += n;
-      g.C += n;
-      g.kflags = K_TO_COL | K_FROM_ROW;
+    chol_inverse<T>(st, ar, n, Z, n, nn, N, n, nn, cnt * P);
+    for (int i = 0; i < cnt; ++i) {
+      const int j = base - 1 - i;
+      T* Ej = E + j * sM;
+      GemmArgs<T> g;
+      g.batch = P;
+      g.m = (!first && together) ? m2 : n; g.n = n; g.k = n; g.opA = OP_N; g.opB = OP_N; g.kflags = K_TO_COL;
+      if (first) { g.A = X; g.lda = n; g.sA = nn; }
+      else { g.A = E + base * sM; g.lda = m2; g.sA = sM * r; }
+      g.B = N + i * nn * P; g.ldb = n; g.sB = nn;
+      g.C = Ej; g.ldc = m2; g.sC = sM * r;
+      g.alpha = one; g.beta = zer; g.site = GS_ZOLO_Q;
       gemm(g, st);
+      if (first) {
+        axpby<T>(st, n, n, 1.0, N + i * nn * P, n, nn, 0.0, Ej + n, m2, sM * r, P);
+      } else if (!together) {
+        g.A += n;
+        g.C += n;
+        g.kflags = K_TO_COL | K_FROM_ROW;
+        gemm(g, st);
+      }
+      gram(Ej, m2, sM * r, G + j * nn, nn * r);
     }
-    gram(Ej, m2, sM * r, G + j * nn, nn * r);
+    base -= cnt;
   }
   scale_terms<T>(st, n, n, pl.sqrtc[0], r, E + n, m2, sM, P);
   {
@@ -185,15 +197,28 @@ static void zolo_first(cudaStream_t st, Arena& ar, const Plan& pl, int n, int P,
     g.alpha = one; g.beta = one; g.site = GS_ZOLO_GRAM2;
     gemm(g, st);
   }
-  T* F = ar.get<T>(nn * P * r);
   minus_eye<T>(st, n, G, n, nn, F, n, nn, P * r);
   T* Y = G;  // the Gram matrices are done with
+  T* D = ar.get<T>(nn * P * r);
   {
-    GemmArgs<T> g;  // Y = Q1 - Q1 (Q1^* Q1 + Q2^* Q2 - I)
+    ReducedScope scope(1u << GS_ZOLO_POLISH, 24);  // E^2 is of order 1e-16
+    GemmArgs<T> g;  // D = E - E E
+    g.batch = P * r;
+    g.m = n; g.n = n; g.k = n; g.opA = OP_N; g.opB = OP_N;
+    g.A = F; g.lda = n; g.sA = nn;
+    g.B = F; g.ldb = n; g.sB = nn;
+    g.Cin = F; g.ldcin = n; g.sCin = nn;
+    g.C = D; g.ldc = n; g.sC = nn;
+    g.alpha = mone; g.beta = one; g.site = GS_ZOLO_POLISH;
+    gemm(g, st);
+  }
+  {
+    ReducedScope scope(1u << GS_ZOLO_POLISH, 40);
+    GemmArgs<T> g;  // Y = Q1 - Q1 D
     g.batch = P * r;
     g.m = n; g.n = n; g.k = n; g.opA = OP_N; g.opB = OP_N;
     g.A = E; g.lda = m2; g.sA = sM;
-    g.B = F; g.ldb = n; g.sB = nn;
+    g.B = D; g.ldb = n; g.sB = nn;
     g.Cin = E; g.ldcin = m2; g.sCin = sM;
     g.C = Y; g.ldc = n; g.sC = nn;
     g.alpha = mone; g.beta = one; g.site = GS_ZOLO_POLISH;
@@ -284,23 +309,8 @@ void zolo_pd(Ctx& cx, Arena& ar, int n, int P, const T* X0, T* W, PolarDiag* pd,
     if (pd) pd->iters += 1;
     // X is well conditioned after the first iteration; with reduced_slices its
     // Gram product and the products with the inverses then keep fewer bits of
-    // their operands, the Cholesky factorizations themselves do not.  The
-    // first iteration's correction E is of order 1e-12 or less: 24 bits of it
-    // reach 1e-19.
-    struct ReducedScope {
-      unsigned sites;
-      int bits;
-      ReducedScope(unsigned s_, int n_) : sites(t_tc.reduced_sites), bits(t_tc.reduced_bits) {
-        t_tc.reduced_sites = s_;
-        t_tc.reduced_bits = n_;
-      }
-      ~ReducedScope() {
-        t_tc.reduced_sites = sites;
-        t_tc.reduced_bits = bits;
-      }
-    };
+    // their operands, the Cholesky factorizations themselves do not.
     if (s == 0) {
-      ReducedScope scope(1u << GS_ZOLO_POLISH, 24);
       zolo_first<T>(st, ar, pl, n, P, X, Xn);
     } else {
       const bool fewer = reduced_slices == 5 || reduced_slices == 6;
@@ -781,9 +791,9 @@ bool is_device_ptr(const void* p) {
 // grows the arena and retries if a bound turns out short.
 size_t polar_bytes(long long n, int P, size_t es, bool tc) {
   const long long nn = n * n, r = R_MAX;
-  // zolo_first's E, G, F and zolo_next's Z, N per term; the recursion's W, V
-  // (n^2 / 4 each at the top, batch P r) and the iterates
-  const long long words = nn * P * (6 * r + 4);
+  // zolo_first's E, G, F, D per term, Z and N of two; the iterates (zolo_next
+  // needs less: Z, N per term and the recursion's W, V, n^2 / 4 each at the top)
+  const long long words = nn * P * (5 * r + 8);
   // residues of the r-term sum on the tensor cores (complex: two real terms)
   const size_t slices = tc ? tc_gemm_bytes(n, n, n, es == 8 ? (int)r : 2) * P : 0;
   return (size_t)(words * es) + slices + 64 * 256;
@@ -791,8 +801,7 @@ size_t polar_bytes(long long n, int P, size_t es, bool tc) {
 
 size_t heig_bytes(long long n, size_t es, bool tc) {
   const long long nn = n * n;
-  long long qr = (long long)ceil_div(n, NB_OUT) * (n + NB_OUT) * NB_OUT +
-                 (long long)ceil_div(n, NB_OUT) * NB_OUT * NB_OUT + (long long)(5 * NB_OUT + (MAX_SUM + 1) * NB_QR) * n;
+  long long qr = 3 * nn;  // P, N and the factor's recursion
   long long leaves = 5 * std::min<long long>(LEAF_MAX, n) * n + 64 * n;  // packed V, T, S, P and FP32 columns: sum sz^2 <= n leaf
   return (size_t)((7 * nn + std::max(qr, leaves)) * es) + polar_bytes(n, 1, es, tc) + (size_t)(3 * n + 2048) * 8 + 64 * 256;
 }

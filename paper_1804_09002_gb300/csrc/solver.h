@@ -3,6 +3,7 @@
 #include <vector>
 
 #include "linalg.h"
+#include "tc_gemm.h"
 #include "profile.h"
 #include "../../include/zolo_csd.h"
 
@@ -66,6 +67,21 @@ struct EigFail {
 const Plan& get_plan(Ctx& cx);
 // device -> host copy on the context stream, then wait for it
 void d2h(Ctx& cx, void* dst, const void* src, size_t bytes);
+
+// Tensor-core products of the call sites in `sites` keep `bits` bits of their
+// operands while this lives (56 is FP64-accurate).
+struct ReducedScope {
+  unsigned sites;
+  int bits;
+  ReducedScope(unsigned s, int b) : sites(t_tc.reduced_sites), bits(t_tc.reduced_bits) {
+    t_tc.reduced_sites = s;
+    t_tc.reduced_bits = b;
+  }
+  ~ReducedScope() {
+    t_tc.reduced_sites = sites;
+    t_tc.reduced_bits = bits;
+  }
+};
 
 // W_p = polar factor of X0_p for p < P (Zolo-pd, Section 5); X0 and W are
 // P consecutive n x n matrices (ld n).  Workspace comes from `ar`.
