@@ -61,8 +61,9 @@ constexpr int JAC_THREADS = 256;
 
 // Column blocks of the FP32 stage of an n-row leaf: nblk (even) blocks of wb
 // columns; a CTA holds two of them in shared memory.  Blocks of 32 columns
-// (16 for columns of more than 512 floats) keep n / 64 SMs busy per leaf
-// and one launch per 32 local rounds.  Leaves of at most 96 rows are one pair
+// keep n / 64 SMs busy per leaf with one launch per 32 local rounds; from 257
+// floats per column on 16 columns are faster (twice the SMs, one column per
+// warp and round).  Leaves of at most 96 rows are one pair
 // of blocks: a single CTA, which then runs every sweep in one launch.
 struct J32Geom {
   int nf;    // floats per column (n, complex 2n)
@@ -75,7 +76,7 @@ __host__ __device__ inline J32Geom j32_geom(int n, bool cplx, int lds) {
   g.nf = cplx ? 2 * n : n;
   g.ldg = (g.nf + 3) & ~3;
   int wmax = J32_SMEM / (8 * lds);
-  const int cap = lds > 512 ? 16 : 32;  // long columns: one per warp fits the registers
+  const int cap = lds >= 384 ? 16 : 32;
   wmax = wmax > cap ? cap : wmax;
   if (n <= 96 && lds <= 512) wmax = (n + 1) / 2;
   const int half = (n + 2 * wmax - 1) / (2 * wmax);
@@ -378,7 +379,7 @@ __global__ void __launch_bounds__(THREADS) j32_kernel(LeafDev L, int pass, int s
       }
     }
   };
-  constexpr int KP = LDS > 512 ? 1 : 2;  // columns of the first block a warp owns across the blocks
+  constexpr int KP = LDS >= 384 ? 1 : 2;  // columns of the first block a warp owns across the blocks
   constexpr bool KEEP = NV <= 8;     // ... in registers
   auto cross = [&]() {
     if constexpr (KEEP) {
