@@ -501,36 +501,26 @@ void launch_panel_smem(cudaStream_t st, int m, int n, int band, T* M, int ldm, l
                                chunk));
 }
 
-// N = L^{-*} of the lower Cholesky factor of an nb x nb block (nb <= 64), one
-// CTA per problem.  Unscaled elimination of [Z | I]: at pivot j every row
-// i > j loses conj(z_ji) / z_jj times row j; then row i of L^{-1} is row i of
-// the right half over sqrt(z_ii).  Column c of the left half is used up to
-// pivot c and column c of the right half from there on, so both share one
-// nb x nb array held in the registers of 1024 threads.  One barrier per pivot:
-// the threads of the next row publish it and its reciprocal pivot as they
-// finish it.  Bound by the FP64 pipe of one SM (a 64-row block: 87 k
-// multiply-adds, 21 us at two per clock) and the chain of 64 pivots.  A warp's
-// FP64 instruction holds its scheduler for 64 clocks, so the rows are spread
-// over 32 warps (two rows each): 77 us a block, where eight warps of eight
-// rows took 104 us and the factor and its inverse by substitution 310 us.
-// (32-row blocks take 30 us but need four more products per 64 columns: no
-// faster.  Complex blocks have 32 rows: 48 us, 64 rows took 237.)
+// N = L^{-*} of the lower Cholesky factor of an nb x nb block (nb <= 32), one
+// CTA per problem, a warp per row and a lane per column.  Unscaled elimination
+// of [Z | I]: at pivot j every row i > j loses conj(z_ji) / z_jj times row j;
+// then row i of L^{-1} is row i of the right half over sqrt(z_ii).  Column c of
+// the left half is used up to pivot c and column c of the right half from
+// there on, so both share one array, an entry per thread.  One barrier per
+// pivot: the warp of the next row publishes it, over its pivot, as it finishes
+// it.  Bound by that chain (27 us a block, 0.8 us a pivot): an FP64 instruction
+// holds its scheduler for 64 clocks, and the reciprocal takes eight in a row.
+// 64 columns at a time (80 us) save four products per pair of blocks and are
+// still 3 % slower over a polar decomposition of n = 1024; the factor and its
+// inverse by substitution took 310 us for 64 columns.
 template <class T>
 __global__ void __launch_bounds__(1024) chol_inv_kernel(int nb, const T* Zall, int ldz, long long sZ, T* Nall, int ldn,
-                                                       long long sN) {
-  constexpr int NB = chol_nb<T>(), TPR = 1024 / NB, EN = NB / TPR;  // threads per row, entries per thread
-  constexpr int RPW = 32 / TPR;                                     // rows of a warp
-  __shared__ T row[2][NB];
-  __shared__ double inv[2];
+                                                        long long sN) {
+  __shared__ T row[2][CHOL_NB], scaled[2][CHOL_NB];
   const T* Zb = Zall + blockIdx.x * sZ;
   T* N = Nall + blockIdx.x * sN;
-  const int tid = threadIdx.x, i = tid / TPR, sub = tid % TPR, iw = i / RPW * RPW;
-  T m[EN];
-#pragma unroll
-  for (int k = 0; k < EN; ++k) {
-    const int c = sub + TPR * k;
-    m[k] = (i < nb && c < nb && i <= c) ? Zb[i + (long long)c * ldz] : zero<T>();
-  }
+  const int i = threadIdx.x >> 5, c = threadIdx.x & 31;
+  T m = (i <= c && c < nb) ? Zb[i + (long long)c * ldz] : zero<T>();
   // 1 / x to rounding: FP32 seed, two Newton steps (NaN unless x > 0)
   auto recip = [](double x) {
     if (!(x > 0.0)) return (double)NAN;
@@ -539,41 +529,28 @@ __global__ void __launch_bounds__(1024) chol_inv_kernel(int nb, const T* Zall, i
     r = fma(r, fma(-x, r, 1.0), r);
     return fma(r, fma(-x, r, 1.0), r);
   };
-  auto publish = [&](int j) {  // by the threads of row j
-#pragma unroll
-    for (int k = 0; k < EN; ++k) {
-      const int c = sub + TPR * k;
-      row[j & 1][c] = m[k];
-      if (c == j) inv[j & 1] = recip(re(m[k]));
-    }
+  // by the warp of row j: the row itself for the factors, and over its pivot,
+  // with 1 / pivot at the pivot's place (column j of the right half)
+  auto publish = [&](int j) {
+    double v = 0.0;
+    if (c == j) v = recip(re(m));
+    v = __shfl_sync(0xffffffffu, v, j);
+    row[j & 1][c] = m;
+    scaled[j & 1][c] = c == j ? from_re<T>(v) : scal(v, m);
   };
   if (i == 0) publish(0);
   for (int j = 0; j + 1 < nb; ++j) {
     __syncthreads();
     if (i > j && i < nb) {
-      const T f = scal(-inv[j & 1], conj_(row[j & 1][i]));
-#pragma unroll
-      for (int k = 0; k < EN; ++k) {
-        if (TPR * k > j && TPR * k + TPR - 1 < iw) continue;  // below the diagonal of the left half
-        const int c = sub + TPR * k;
-        m[k] = c == j ? f : fmac(f, row[j & 1][c], m[k]);
-      }
+      const T nf = scal(-1.0, conj_(row[j & 1][i]));
+      m = fmac(nf, scaled[j & 1][c], c == j ? zero<T>() : m);
       if (i == j + 1) publish(i);
     }
   }
   if (i < nb) {
-    double d = 0.0;
-#pragma unroll
-    for (int k = 0; k < EN; ++k)
-      if (sub + TPR * k == i) d = re(m[k]);
-    d = __shfl_sync(__activemask(), d, (tid & 31) / TPR * TPR + i % TPR);
+    const double d = __shfl_sync(0xffffffffu, re(m), i);
     const double s = d > 0.0 ? 1.0 / sqrt(d) : (double)NAN;
-#pragma unroll
-    for (int k = 0; k < EN; ++k) {
-      const int c = sub + TPR * k;
-      if (c < i) N[c + (long long)i * ldn] = scal(s, conj_(m[k]));
-      else if (c == i) N[c + (long long)i * ldn] = from_re<T>(s);
-    }
+    if (c <= i) N[c + (long long)i * ldn] = c < i ? scal(s, conj_(m)) : from_re<T>(s);
   }
 }
 
@@ -620,7 +597,7 @@ void qr_panel(cudaStream_t st, int m, int n, int band, T* M, int ldm, long long 
 template <class T>
 void chol_inv_block(cudaStream_t st, int nb, const T* Z, int ldz, long long sZ, T* N, int ldn, long long sN,
                     int batch) {
-  if (nb > chol_nb<T>()) throw CudaFail{cudaErrorInvalidValue, __FILE__, __LINE__};
+  if (nb > CHOL_NB) throw CudaFail{cudaErrorInvalidValue, __FILE__, __LINE__};
   ProfToken tok = prof_begin(st);
   chol_inv_kernel<T><<<batch, 1024, 0, st>>>(nb, Z, ldz, sZ, N, ldn, sN);
   ZCSD_LAUNCH();

@@ -219,13 +219,12 @@ void qr_form_q(cudaStream_t st, Arena& ar, const QRStore<T>& q, T* E, int lde, l
 template <class T>
 static void chol_inv_rec(cudaStream_t st, Arena& ar, int c0, int c1, T* Z, int ldz, long long sZ, T* N, int ldn,
                          long long sN, int batch) {
-  constexpr int NB = chol_nb<T>();
   const int w = c1 - c0;
-  if (w <= NB) {
+  if (w <= CHOL_NB) {
     chol_inv_block<T>(st, w, Z + c0 + (long long)c0 * ldz, ldz, sZ, N + c0 + (long long)c0 * ldn, ldn, sN, batch);
     return;
   }
-  const int mid = c0 + ceil_div(w / 2, NB) * NB, w1 = mid - c0, w2 = c1 - mid;
+  const int mid = c0 + ceil_div(w / 2, CHOL_NB) * CHOL_NB, w1 = mid - c0, w2 = c1 - mid;
   const T one = from_re<T>(1.0), mone = from_re<T>(-1.0), zer = zero<T>();
   chol_inv_rec(st, ar, c0, mid, Z, ldz, sZ, N, ldn, sN, batch);
   const size_t mk = ar.mark();

@@ -115,9 +115,9 @@ template <class T> void randn(cudaStream_t st, int m, int n, T* X, int ldx, unsi
 template <class T> void qr_panel(cudaStream_t st, int m, int n, int band, T* M, int ldm, long long sM,
                                  int k0, int nb, T* Y, int ldy, long long sY, T* Tf, long long sT, int batch);
 // N = R^{-1} (upper triangular; only its upper triangle is written) of the
-// upper Cholesky factor R^* R = Z of nb x nb blocks, nb <= chol_nb, from Z's
+// upper Cholesky factor R^* R = Z of nb x nb blocks, nb <= CHOL_NB, from Z's
 // upper triangle; NaN where Z is not positive definite.
-template <class T> __host__ __device__ constexpr int chol_nb() { return sizeof(T) == 8 ? 64 : 32; }
+constexpr int CHOL_NB = 32;
 template <class T> void chol_inv_block(cudaStream_t st, int nb, const T* Z, int ldz, long long sZ, T* N, int ldn,
                                        long long sN, int batch);
 }  // namespace zcsd
