@@ -112,7 +112,7 @@ void d2h(Ctx& cx, void* dst, const void* src, size_t bytes) {
 //     for every X, so there is no pivot to check.
 // Two terms follow from each basis, 1 / rho = 4.7e3 and 2.2e7, so that the
 // chain is four factorizations of two problems long (eight of one leave more
-// SMs idle: the factorization of n = 1024 is a chain of 16 blocks of 77 us).
+// SMs idle: a factorization is a chain of 32-column blocks).
 // Each step leaves a departure E = Q1^* Q1 + Q2^* Q2 - I of order u / rho, 1e-8
 // at most, which does not grow along the chain; the term of the exact basis is
 // Q1 (I + E)^{-1} Q2^*, two more products up to E^3.  The result is as accurate
@@ -198,29 +198,37 @@ static void zolo_first(cudaStream_t st, Arena& ar, const Plan& pl, int n, int P,
     gemm(g, st);
   }
   minus_eye<T>(st, n, G, n, nn, F, n, nn, P * r);
+  // Y = Q1 - Q1 (E - E^2): the first term of each step has E of order 1e-12,
+  // where E^2 and all but 24 bits of E are below rounding; the second, 1e-8,
+  // keeps 40 bits and E^2.  With an even number of terms these are every other
+  // problem of the batch.
   T* Y = G;  // the Gram matrices are done with
-  T* D = ar.get<T>(nn * P * r);
+  const bool split = r % 2 == 0;
+  const int half = split ? P * r / 2 : P * r;
+  const long long hop = split ? 2 : 1;
+  T* D = ar.get<T>(nn * half);
   {
     ReducedScope scope(1u << GS_ZOLO_POLISH, 24);  // E^2 is of order 1e-16
     GemmArgs<T> g;  // D = E - E E
-    g.batch = P * r;
+    g.batch = half;
     g.m = n; g.n = n; g.k = n; g.opA = OP_N; g.opB = OP_N;
-    g.A = F; g.lda = n; g.sA = nn;
-    g.B = F; g.ldb = n; g.sB = nn;
-    g.Cin = F; g.ldcin = n; g.sCin = nn;
+    g.A = F; g.lda = n; g.sA = hop * nn;
+    g.B = F; g.ldb = n; g.sB = hop * nn;
+    g.Cin = F; g.ldcin = n; g.sCin = hop * nn;
     g.C = D; g.ldc = n; g.sC = nn;
     g.alpha = mone; g.beta = one; g.site = GS_ZOLO_POLISH;
     gemm(g, st);
   }
-  {
-    ReducedScope scope(1u << GS_ZOLO_POLISH, 40);
-    GemmArgs<T> g;  // Y = Q1 - Q1 D
-    g.batch = P * r;
+  for (int odd = 0; odd < (split ? 2 : 1); ++odd) {
+    ReducedScope scope(1u << GS_ZOLO_POLISH, odd ? 24 : 40);
+    GemmArgs<T> g;
+    g.batch = half;
     g.m = n; g.n = n; g.k = n; g.opA = OP_N; g.opB = OP_N;
-    g.A = E; g.lda = m2; g.sA = sM;
-    g.B = D; g.ldb = n; g.sB = nn;
-    g.Cin = E; g.ldcin = m2; g.sCin = sM;
-    g.C = Y; g.ldc = n; g.sC = nn;
+    g.A = E + odd * sM; g.lda = m2; g.sA = hop * sM;
+    if (odd) { g.B = F + nn; g.ldb = n; g.sB = hop * nn; }
+    else { g.B = D; g.ldb = n; g.sB = nn; }
+    g.Cin = E + odd * sM; g.ldcin = m2; g.sCin = hop * sM;
+    g.C = Y + odd * nn; g.ldc = n; g.sC = hop * nn;
     g.alpha = mone; g.beta = one; g.site = GS_ZOLO_POLISH;
     gemm(g, st);
   }
