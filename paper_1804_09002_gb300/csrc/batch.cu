@@ -17,9 +17,12 @@
 //    products on the padded V, then one CTA per instance sorts its angles
 //    and writes its columns into the packed outputs.
 //
-// Everything between the input and the output buffers is on one stream with
-// no host synchronisation, so the whole batch is captured once into a CUDA
-// graph and replayed.  An autotuner picks the bucket granularity and, per
+// Everything between the input and the output buffers runs with no host
+// synchronisation, so the whole batch is captured once into a CUDA graph and
+// replayed.  A bucket is a chain of small launches that leaves most SMs idle,
+// and buckets share nothing but read-only inputs, so they run side by side on
+// up to MAX_LANES streams, each with its own part of the workspace (48
+// instances of 16..256 rows in 16 buckets: 36 ms on one stream).  An autotuner picks the bucket granularity and, per
 // bucket, the product engine (FP64-pipe tiles or the tensor-core kernel) by
 // timing each candidate once on the caller's data.
 #include <algorithm>
@@ -37,12 +40,15 @@ namespace zcsd {
 namespace {
 
 constexpr int BATCH_MAX_N = 1024;
+constexpr int MAX_LANES = 8;
+constexpr size_t LANE_BYTES = (size_t)48 << 30;  // workspace of all lanes together, where more than one needs it
 constexpr int BATCH_SWEEPS = 30;  // FP64 Jacobi sweeps at most of a leaf that the refinement leaves open
 
 struct Bucket {
   int nb = 0;                    // padded size
   std::vector<int> inst;         // instance indices
   bool tc = false;               // products on the tensor cores
+  int lane = 0;                  // stream and workspace part it runs on
   // device tables (persistent region): per bucket problem p (instance inst[p])
   int* dn = nullptr;             // n_i
   long long* doff = nullptr;     // element offset of instance i in the packed matrices
@@ -223,8 +229,12 @@ struct csd_batch {
   bool tuned = false;
   double ws_scale = 1.0;                // grows when a run overflows the arena
   size_t run_need = 0;                  // arena bytes a run was seen to need
-  cudaStream_t stream = nullptr;        // the plan's own stream (tuning, capture, replay)
+  cudaStream_t stream = nullptr;        // the plan's own stream (tuning, capture, replay): lane 0
   cudaEvent_t ev = nullptr;
+  int lanes = 1;
+  cudaStream_t side[MAX_LANES] = {};    // lanes 1 .. lanes - 1
+  cudaEvent_t side_ev[MAX_LANES] = {};
+  size_t lane_off[MAX_LANES + 1] = {};  // workspace parts, from persist_bytes
 };
 
 namespace {
@@ -274,15 +284,37 @@ int build_buckets(csd_batch* b, int gran) {
     pbytes += bk.inst.size() * 128 + leaf_table_bytes(sz, false) + 16 * 256;
   }
   pbytes += (size_t)b->count * 16 + 4 * 256 + (1 << 20);
-  size_t run = 0;
+  std::vector<size_t> need;
   for (auto& bk : b->buckets) {
     long long vt = 0;
     for (int i : bk.inst) vt += (long long)b->n[i] * b->n[i];
     bk.leaves.vtot = vt;
-    run = std::max(run, bucket_bytes(bk));
+    need.push_back(std::max((size_t)((double)bucket_bytes(bk) * b->ws_scale), b->run_need));
   }
   b->persist_bytes = (pbytes + 255) & ~(size_t)255;
-  b->ws_bytes = b->persist_bytes + std::max((size_t)((double)run * b->ws_scale), b->run_need);
+  // lanes: the largest buckets first, each to the lane with the least work so
+  // far (a bucket's time grows with its size, hardly with its instances); as
+  // many lanes as fit LANE_BYTES
+  std::vector<int> order((int)b->buckets.size());
+  for (size_t k = 0; k < order.size(); ++k) order[k] = (int)k;
+  std::sort(order.begin(), order.end(), [&](int x, int y) { return b->buckets[x].nb > b->buckets[y].nb; });
+  for (b->lanes = std::min<int>(MAX_LANES, (int)b->buckets.size());; --b->lanes) {
+    size_t bytes[MAX_LANES] = {}, total = 0;
+    double load[MAX_LANES] = {};
+    for (int k : order) {
+      const int l = (int)(std::min_element(load, load + b->lanes) - load);
+      b->buckets[k].lane = l;
+      load[l] += b->buckets[k].nb + 32.0;
+      bytes[l] = std::max(bytes[l], (need[k] + 255) & ~(size_t)255);
+    }
+    for (int l = 0; l < b->lanes; ++l) {
+      b->lane_off[l] = total;
+      total += bytes[l];
+    }
+    b->lane_off[b->lanes] = total;
+    if (b->lanes == 1 || total <= LANE_BYTES) break;
+  }
+  b->ws_bytes = b->persist_bytes + b->lane_off[b->lanes];
   if (cudaMalloc((void**)&b->ws, b->ws_bytes) != cudaSuccess) {
     cudaGetLastError();
     b->ws = nullptr;
@@ -331,14 +363,33 @@ int build_buckets(csd_batch* b, int gran) {
   return CSD_OK;
 }
 
-// The whole batch on the context stream (capturable: no host sync).
+struct StreamSwap {
+  Ctx& c;
+  cudaStream_t prev;
+  StreamSwap(Ctx& c_, cudaStream_t s) : c(c_), prev(c_.stream) { c.stream = s; }
+  ~StreamSwap() { c.stream = prev; }
+};
+
+// The whole batch, forked from and joined to the context stream (capturable:
+// no host sync).
 void run_all(csd_batch* b, const double* A1, const double* A2, double* U1, double* U2, double* V1, double* theta) {
   Ctx& cx = *b->cx;
-  Arena ar;
-  ar.base = b->ws + b->persist_bytes;
-  ar.cap = b->ws_bytes - b->persist_bytes;
-  for (size_t k = 0; k < b->buckets.size(); ++k)
-    run_bucket(cx, ar, b->buckets[k], A1, A2, U1, U2, V1, theta, b->dstatus, b->dinst + b->inst_off[k], b->tc_err);
+  ZCSD_CUDA(cudaEventRecord(b->ev, cx.stream));
+  for (int l = 1; l < b->lanes; ++l) ZCSD_CUDA(cudaStreamWaitEvent(b->side[l], b->ev, 0));
+  for (int l = 0; l < b->lanes; ++l) {
+    StreamSwap lane(cx, l ? b->side[l] : cx.stream);
+    for (size_t k = 0; k < b->buckets.size(); ++k) {
+      if (b->buckets[k].lane != l) continue;
+      Arena ar;
+      ar.base = b->ws + b->persist_bytes + b->lane_off[l];
+      ar.cap = b->lane_off[l + 1] - b->lane_off[l];
+      run_bucket(cx, ar, b->buckets[k], A1, A2, U1, U2, V1, theta, b->dstatus, b->dinst + b->inst_off[k], b->tc_err);
+    }
+  }
+  for (int l = 1; l < b->lanes; ++l) {
+    ZCSD_CUDA(cudaEventRecord(b->side_ev[l], b->side[l]));
+    ZCSD_CUDA(cudaStreamWaitEvent(cx.stream, b->side_ev[l], 0));
+  }
 }
 
 // Per bucket engine choice, then the granularity with the smallest total.
@@ -443,18 +494,16 @@ int csd_batch_run(csd_batch* b, const double* A1, const double* A2, double* U1, 
   // stream other than the legacy default one), ordered after the work
   // already queued on the context's stream and before whatever follows it
   if (!b->stream) {
-    if (cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming) != cudaSuccess) {
+    bool ok = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) == cudaSuccess &&
+              cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming) == cudaSuccess;
+    for (int l = 1; l < MAX_LANES; ++l)
+      ok = ok && cudaStreamCreateWithFlags(&b->side[l], cudaStreamNonBlocking) == cudaSuccess &&
+           cudaEventCreateWithFlags(&b->side_ev[l], cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) {
       cudaGetLastError();
       return CSD_ERR_CUDA;
     }
   }
-  struct StreamSwap {
-    Ctx& c;
-    cudaStream_t prev;
-    StreamSwap(Ctx& c_, cudaStream_t s) : c(c_), prev(c_.stream) { c.stream = s; }
-    ~StreamSwap() { c.stream = prev; }
-  };
   if (cudaEventRecord(b->ev, cx.stream) != cudaSuccess || cudaStreamWaitEvent(b->stream, b->ev, 0) != cudaSuccess) {
     cudaGetLastError();
     return CSD_ERR_CUDA;
@@ -498,6 +547,7 @@ int csd_batch_run(csd_batch* b, const double* A1, const double* A2, double* U1, 
       if (g) cudaGraphDestroy(g);
     }
     cudaStreamSynchronize(cx.stream);
+    for (int l = 1; l < MAX_LANES; ++l) cudaStreamSynchronize(b->side[l]);
     cudaGetLastError();
     if (attempt >= 6) return CSD_ERR_INTERNAL;
     b->ws_scale *= 2.0;
@@ -529,6 +579,13 @@ int csd_batch_destroy(csd_batch* b) {
   if (!b) return CSD_OK;
   cudaSetDevice(b->cx->device);
   if (b->stream) cudaStreamSynchronize(b->stream);
+  for (int l = 1; l < MAX_LANES; ++l) {
+    if (b->side[l]) {
+      cudaStreamSynchronize(b->side[l]);
+      cudaStreamDestroy(b->side[l]);
+    }
+    if (b->side_ev[l]) cudaEventDestroy(b->side_ev[l]);
+  }
   free_plan_ws(b);
   if (b->ev) cudaEventDestroy(b->ev);
   if (b->stream) cudaStreamDestroy(b->stream);

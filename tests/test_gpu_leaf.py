@@ -55,3 +55,24 @@ def test_leaf_eigendecomposition(B, n, cplx, tc, kind):
     assert np.max(np.abs(lam - np.linalg.eigvalsh(M))) <= 50 * n * U * nb
     assert np.linalg.norm(M @ V - V * lam) <= 50 * n * U * nb
     assert np.linalg.norm(V.conj().T @ V - np.eye(n), 2) <= 50 * n * U
+
+
+@pytest.mark.parametrize("n,cplx,tc", [(65, False, False), (150, True, False), (330, False, True), (300, True, True)])
+@pytest.mark.parametrize("kind", ["gauss", "repeated"])
+def test_splits_into_small_leaves(B, n, cplx, tc, kind):
+    """Zolo-eig's splits on small blocks (leaves of at most 32 rows): the two
+    bases from one inverse Cholesky factor, padded groups of different sizes."""
+    M = _matrix(kind, n, cplx)
+    ctx = B.Context(0)
+    try:
+        ctx.set_tensor_cores(tc)
+        ctx.set_eig_leaf(32)
+        lam, V, info = ctx.heig(to_dev(M))
+        lam, V = to_host(lam), to_host(V)
+    finally:
+        ctx.close()
+    assert info["eig_splits"] >= 1
+    nb = np.linalg.norm(M, 2)
+    assert np.max(np.abs(lam - np.linalg.eigvalsh(M))) <= 50 * n * U * nb
+    assert np.linalg.norm(M @ V - V * lam) <= 50 * n * U * nb
+    assert np.linalg.norm(V.conj().T @ V - np.eye(n), 2) <= 50 * n * U
