@@ -22,9 +22,10 @@
 // replayed.  A bucket is a chain of small launches that leaves most SMs idle,
 // and buckets share nothing but read-only inputs, so they run side by side on
 // up to MAX_LANES streams, each with its own part of the workspace (48
-// instances of 16..256 rows in 16 buckets: 36 ms on one stream).  An autotuner picks the bucket granularity and, per
-// bucket, the product engine (FP64-pipe tiles or the tensor-core kernel) by
-// timing each candidate once on the caller's data.
+// instances of 16..256 rows in 16 buckets: 36.4 ms on one stream, 26.5 ms).  An
+// autotuner picks the bucket granularity and, per bucket, the product engine
+// (FP64-pipe tiles or the tensor-core kernel) by timing each candidate once on
+// the caller's data.
 #include <algorithm>
 #include <cstring>
 #include <map>
@@ -294,7 +295,8 @@ int build_buckets(csd_batch* b, int gran) {
   b->persist_bytes = (pbytes + 255) & ~(size_t)255;
   // lanes: the largest buckets first, each to the lane with the least work so
   // far (a bucket's time grows with its size, hardly with its instances); as
-  // many lanes as fit LANE_BYTES
+  // many lanes as fit LANE_BYTES and the memory that is free (one lane needs no
+  // more than the largest bucket)
   std::vector<int> order((int)b->buckets.size());
   for (size_t k = 0; k < order.size(); ++k) order[k] = (int)k;
   std::sort(order.begin(), order.end(), [&](int x, int y) { return b->buckets[x].nb > b->buckets[y].nb; });
@@ -312,13 +314,13 @@ int build_buckets(csd_batch* b, int gran) {
       total += bytes[l];
     }
     b->lane_off[b->lanes] = total;
-    if (b->lanes == 1 || total <= LANE_BYTES) break;
-  }
-  b->ws_bytes = b->persist_bytes + b->lane_off[b->lanes];
-  if (cudaMalloc((void**)&b->ws, b->ws_bytes) != cudaSuccess) {
+    if (b->lanes > 1 && total > LANE_BYTES) continue;
+    b->ws_bytes = b->persist_bytes + total;
+    if (cudaMalloc((void**)&b->ws, b->ws_bytes) == cudaSuccess) break;
     cudaGetLastError();
     b->ws = nullptr;
-    return CSD_ERR_ALLOC;
+    b->ws_bytes = 0;
+    if (b->lanes == 1) return CSD_ERR_ALLOC;
   }
   Ctx& cx = *b->cx;
   Arena per;
