@@ -21,10 +21,15 @@ constexpr int NT = 256;
 // Output tile BM x BN, RM x RN outputs per thread (256 threads), k-step BK.
 // The next k-step's operands are loaded into registers before the current
 // one is consumed (not where a thread's complex 4 x 4 outputs fill them).
+// Tiles of fewer than 256 outputs share every k-step among KG groups of
+// threads, whose sums are added at the end.  A warp instruction holds its
+// scheduler's FP64 lanes for 64 clocks, so nothing is issued that can be left
+// out: unit weights and alpha, rows and columns beyond the edge.
 template <class T, int OPA, int OPB, int BM, int BN, int RM, int RN, int BK>
 __global__ void __launch_bounds__(NT, 2) gemm_kernel(GemmArgs<T> g) {
   constexpr int TX = BM / RM, TY = BN / RN;  // thread grid over the tile
-  static_assert(TX * TY == NT, "256 threads");
+  constexpr int KG = NT / (TX * TY);
+  static_assert(TX * TY * KG == NT && TX * TY % 32 == 0 && BK % KG == 0, "256 threads, whole warps per group");
   constexpr int LA = BM * BK / NT, LB = BN * BK / NT;
   constexpr bool AHEAD = sizeof(T) == 8 || RM * RN < 16;
   const int z = blockIdx.z;
@@ -46,7 +51,10 @@ __global__ void __launch_bounds__(NT, 2) gemm_kernel(GemmArgs<T> g) {
   __shared__ T As[BK][BM + 1];
   __shared__ T Bs[BK][BN + 1];
   const int tid = threadIdx.x;
-  const int tx = tid % TX, ty = tid / TX;
+  const int tx = tid % TX, ty = tid % (TX * TY) / TX, kg = tid / (TX * TY);
+  // outputs inside the matrix: row blocks of the tile, column blocks of the warp
+  const int rows = min(RM, (g.m - m0 + TX - 1) / TX);
+  const int cols = min(RN, (g.n - n0 - (tid & ~31) % (TX * TY) / TX + TY - 1) / TY);
   T acc[RM][RN];
 #pragma unroll
   for (int i = 0; i < RM; ++i)
@@ -76,7 +84,7 @@ __global__ void __launch_bounds__(NT, 2) gemm_kernel(GemmArgs<T> g) {
           if (OPA == OP_C) v = conj_(v);
         }
       }
-      va[s] = scal(wj, v);
+      va[s] = wj != 1.0 ? scal(wj, v) : v;
     }
 #pragma unroll
     for (int s = 0; s < LB; ++s) {
@@ -112,7 +120,8 @@ __global__ void __launch_bounds__(NT, 2) gemm_kernel(GemmArgs<T> g) {
     __syncthreads();
     if (AHEAD && it + 1 < total) fetch(it + 1);
 #pragma unroll
-    for (int k = 0; k < BK; ++k) {
+    for (int kk = 0; kk < BK; kk += KG) {
+      const int k = kk + kg;
       T a[RM], bb[RN];
 #pragma unroll
       for (int i = 0; i < RM; ++i) a[i] = As[k][tx + TX * i];
@@ -121,13 +130,24 @@ __global__ void __launch_bounds__(NT, 2) gemm_kernel(GemmArgs<T> g) {
 #pragma unroll
       for (int i = 0; i < RM; ++i)
 #pragma unroll
-        for (int j = 0; j < RN; ++j) acc[i][j] = fmac(a[i], bb[j], acc[i][j]);
+        for (int j = 0; j < RN; ++j)
+          if (i < rows && j < cols) acc[i][j] = fmac(a[i], bb[j], acc[i][j]);
     }
     __syncthreads();
+  }
+  if constexpr (KG > 1) {
+    static_assert(RM == 1 && RN == 1 && (KG - 1) * BM * BN <= BK * (BM + 1), "sums of the groups fit As");
+    T* sums = &As[0][0];
+    if (kg > 0) sums[tid - BM * BN] = acc[0][0];
+    __syncthreads();
+    if (kg > 0) return;
+#pragma unroll
+    for (int s = 0; s < KG - 1; ++s) acc[0][0] = add(acc[0][0], sums[tid + s * BM * BN]);
   }
   // ---- epilogue
   T* C = g.C + z * g.sC;
   const T* Cin = g.Cin ? g.Cin + (b / g.bdivC) * g.sCin : nullptr;
+  const bool unit = re(g.alpha) == 1.0 && im(g.alpha) == 0.0;
   const bool use_beta = Cin && ks == 0 && (re(g.beta) != 0.0 || im(g.beta) != 0.0);
 #pragma unroll
   for (int j = 0; j < RN; ++j) {
@@ -137,7 +157,7 @@ __global__ void __launch_bounds__(NT, 2) gemm_kernel(GemmArgs<T> g) {
     for (int i = 0; i < RM; ++i) {
       const int gi = m0 + tx + TX * i;
       if (gi >= g.m) continue;
-      T v = mul(g.alpha, acc[i][j]);
+      T v = unit ? acc[i][j] : mul(g.alpha, acc[i][j]);
       if (use_beta) v = fmac(g.beta, Cin[gi + (long long)gj * g.ldcin], v);
       C[gi + (long long)gj * g.ldc] = v;
     }
@@ -150,9 +170,12 @@ __global__ void __launch_bounds__(NT, 2) gemm_kernel(GemmArgs<T> g) {
 // BM x BN outputs.  128^3 (two problems): 64 x 64 tiles on 8 SMs take 130 us,
 // 16 x 16 tiles 9 us.  Large outputs keep 64 x 64 (32 x 128 for m <= 32),
 // which read each operand least often; a smaller tile has to win by 10 %.
+// The products between the 32-column blocks of an inverse Cholesky factor fill
+// the chip with 8 x 8 tiles only (csd n = 64 1.65 -> 1.53 ms, n = 201 6.60 ->
+// 6.13, polar n = 2048 42.8 -> 41.1, together with what the kernel leaves out).
 // A product in place needs one tile over the whole of what it overwrites.
-enum GemmTile { TILE_64 = 0, TILE_32x128, TILE_32, TILE_16, TILES };
-constexpr int TILE_M[TILES] = {64, 32, 32, 16}, TILE_N[TILES] = {64, 128, 32, 16};
+enum GemmTile { TILE_64 = 0, TILE_32x128, TILE_32, TILE_16, TILE_16x8, TILE_8, TILES };
+constexpr int TILE_M[TILES] = {64, 32, 32, 16, 16, 8}, TILE_N[TILES] = {64, 128, 32, 16, 8, 8};
 
 template <class T>
 int pick_tile(const GemmArgs<T>& g) {
@@ -180,7 +203,9 @@ void gemm_launch(const GemmArgs<T>& g, int tile, cudaStream_t st) {
     case TILE_64: gemm_kernel<T, OPA, OPB, 64, 64, 4, 4, 16><<<grid, NT, 0, st>>>(g); break;
     case TILE_32x128: gemm_kernel<T, OPA, OPB, 32, 128, 4, 4, 16><<<grid, NT, 0, st>>>(g); break;
     case TILE_32: gemm_kernel<T, OPA, OPB, 32, 32, 2, 2, 16><<<grid, NT, 0, st>>>(g); break;
-    default: gemm_kernel<T, OPA, OPB, 16, 16, 1, 1, 32><<<grid, NT, 0, st>>>(g); break;
+    case TILE_16: gemm_kernel<T, OPA, OPB, 16, 16, 1, 1, 32><<<grid, NT, 0, st>>>(g); break;
+    case TILE_16x8: gemm_kernel<T, OPA, OPB, 16, 8, 1, 1, 32><<<grid, NT, 0, st>>>(g); break;
+    default: gemm_kernel<T, OPA, OPB, 8, 8, 1, 1, 32><<<grid, NT, 0, st>>>(g); break;
   }
 }
 
