@@ -499,23 +499,15 @@ __global__ void theta_lambda_kernel(int n, const double* lam, double* th) {
   }
 }
 
-// rank of each key among all keys (ties by index): perm[rank] = index.
-// NaN keys order after +inf, so the ranks always form a permutation.
-__device__ inline double sort_key(double v) { return isnan(v) ? INFINITY : v; }
-
-__global__ void sort_perm_kernel(int n, const double* key, int* perm) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const double v = sort_key(key[i]);
-    const bool vnan = isnan(key[i]);
-    int rank = 0;
-    for (int k = 0; k < n; ++k) {
-      const double w = sort_key(key[k]);
-      const bool wnan = isnan(key[k]);
-      const bool before = (w < v) || (w == v && (wnan == vnan ? k < i : !wnan));
-      rank += before;
-    }
-    perm[rank] = i;
-  }
+// rank of each key among all keys (ties by index): perm[rank] = index, a warp
+// per key.  NaN keys order after +inf, so the ranks always form a permutation.
+// A thread per key compared on the FP64 pipe of n / 256 SMs: 303 us at n =
+// 1024.
+__global__ void __launch_bounds__(256) sort_perm_kernel(int n, const double* key, int* perm) {
+  const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (i >= n) return;
+  const int r = warp_rank(key, n, i);
+  if ((threadIdx.x & 31) == 0) perm[r] = i;
 }
 
 template <class T>
@@ -620,7 +612,7 @@ void theta_from_lambda(cudaStream_t st, int n, const double* lam, double* theta)
 
 void sort_perm(cudaStream_t st, int n, const double* key, int* perm) {
   if (n <= 0) return;
-  sort_perm_kernel<<<ceil_div(n, 256), 256, 0, st>>>(n, key, perm);
+  sort_perm_kernel<<<ceil_div(n, 8), 256, 0, st>>>(n, key, perm);
   ZCSD_LAUNCH();
 }
 

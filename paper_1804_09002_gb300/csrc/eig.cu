@@ -91,21 +91,13 @@ __global__ void blk_diag(const T* B, int n, const int* off, const int* sz, doubl
     d[o + i] = re(B[(long long)(o + i) * (n + 1)]);
 }
 
-// out[p] = lower median of d[off_p .. off_p + sz_p) (rank counting, one CTA)
-__global__ void blk_median(const double* d, const int* off, const int* sz, double* out) {
-  const int p = blockIdx.x, m = sz[p];
+// out[p] = lower median of d[off_p .. off_p + sz_p), by rank counting: a warp
+// per entry (one CTA per block on the FP64 pipe: 3.3 ms at 3000 rows)
+__global__ void __launch_bounds__(256) blk_median(const double* d, const int* off, const int* sz, double* out) {
+  const int p = blockIdx.y, m = sz[p], i = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (i >= m) return;
   const double* dp = d + off[p];
-  const int want = (m - 1) / 2;
-  for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    const double v = dp[i];
-    int less = 0, eq_before = 0;
-    for (int k = 0; k < m; ++k) {
-      const double w = dp[k];
-      less += (w < v);
-      eq_before += (w == v && k < i);
-    }
-    if (less + eq_before == want) out[p] = v;
-  }
+  if (warp_rank(dp, m, i) == (m - 1) / 2 && (threadIdx.x & 31) == 0) out[p] = dp[i];
 }
 
 // X_p = diag((B_p - s_p I) / xn_p, I), nb x nb, B_p the sz_p block at (off_p, off_p)
@@ -307,7 +299,7 @@ void heig_impl(Ctx& cx, Arena& ar, int n, const T* Bin, int ldb, double* lam, T*
       const int* dsz = upload(ar, st, sz);
       blk_diag<T><<<dim3(8, P), 256, 0, st>>>(Bw, n, doff, dsz, dvals);
       ZCSD_LAUNCH();
-      blk_median<<<P, 256, 0, st>>>(dvals, doff, dsz, d);
+      blk_median<<<dim3(ceil_div(*std::max_element(sz.begin(), sz.end()), 8), P), 256, 0, st>>>(dvals, doff, dsz, d);
       ZCSD_LAUNCH();
       const std::vector<double> h = download(cx, d, P);
       for (int p = 0; p < P; ++p) {
