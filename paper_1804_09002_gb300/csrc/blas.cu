@@ -35,6 +35,7 @@ __global__ void __launch_bounds__(NT, 2) gemm_kernel(GemmArgs<T> g) {
   const int z = blockIdx.z;
   const int b = z / g.ksplit, ks = z % g.ksplit;
   const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
+  chain_wait();
   if (g.uplo == 1 && m0 > n0 + BN - 1) return;
   if (g.uplo == 2 && n0 > m0 + BM - 1) return;
   int kb = 0, ke = g.k;
@@ -145,6 +146,7 @@ __global__ void __launch_bounds__(NT, 2) gemm_kernel(GemmArgs<T> g) {
     for (int s = 0; s < KG - 1; ++s) acc[0][0] = add(acc[0][0], sums[tid + s * BM * BN]);
   }
   // ---- epilogue
+  chain_next();
   T* C = g.C + z * g.sC;
   const T* Cin = g.Cin ? g.Cin + (b / g.bdivC) * g.sCin : nullptr;
   const bool unit = re(g.alpha) == 1.0 && im(g.alpha) == 0.0;
@@ -200,12 +202,12 @@ template <class T, int OPA, int OPB>
 void gemm_launch(const GemmArgs<T>& g, int tile, cudaStream_t st) {
   const dim3 grid(ceil_div(g.m, TILE_M[tile]), ceil_div(g.n, TILE_N[tile]), g.batch * g.ksplit);
   switch (tile) {
-    case TILE_64: gemm_kernel<T, OPA, OPB, 64, 64, 4, 4, 16><<<grid, NT, 0, st>>>(g); break;
-    case TILE_32x128: gemm_kernel<T, OPA, OPB, 32, 128, 4, 4, 16><<<grid, NT, 0, st>>>(g); break;
-    case TILE_32: gemm_kernel<T, OPA, OPB, 32, 32, 2, 2, 16><<<grid, NT, 0, st>>>(g); break;
-    case TILE_16: gemm_kernel<T, OPA, OPB, 16, 16, 1, 1, 32><<<grid, NT, 0, st>>>(g); break;
-    case TILE_16x8: gemm_kernel<T, OPA, OPB, 16, 8, 1, 1, 32><<<grid, NT, 0, st>>>(g); break;
-    default: gemm_kernel<T, OPA, OPB, 8, 8, 1, 1, 32><<<grid, NT, 0, st>>>(g); break;
+    case TILE_64: launch_chained(gemm_kernel<T, OPA, OPB, 64, 64, 4, 4, 16>, grid, NT, 0, st, g); break;
+    case TILE_32x128: launch_chained(gemm_kernel<T, OPA, OPB, 32, 128, 4, 4, 16>, grid, NT, 0, st, g); break;
+    case TILE_32: launch_chained(gemm_kernel<T, OPA, OPB, 32, 32, 2, 2, 16>, grid, NT, 0, st, g); break;
+    case TILE_16: launch_chained(gemm_kernel<T, OPA, OPB, 16, 16, 1, 1, 32>, grid, NT, 0, st, g); break;
+    case TILE_16x8: launch_chained(gemm_kernel<T, OPA, OPB, 16, 8, 1, 1, 32>, grid, NT, 0, st, g); break;
+    default: launch_chained(gemm_kernel<T, OPA, OPB, 8, 8, 1, 1, 32>, grid, NT, 0, st, g); break;
   }
 }
 

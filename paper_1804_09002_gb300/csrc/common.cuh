@@ -105,6 +105,34 @@ void count_launch();
     ZCSD_CUDA(cudaGetLastError());     \
   } while (0)
 
+#ifdef __CUDACC__
+// Kernels of the long chains of short launches (small products, Cholesky
+// blocks, Jacobi rounds) are launched while their predecessor ends: every
+// thread that touches memory first waits for all of the predecessor
+// (chain_wait), and a CTA that has only its results left to write lets the
+// successor's CTAs in (chain_next; a CTA that exits counts too).  A kernel
+// launched without the attribute waits as ever, and so does whatever follows a
+// chained kernel without it.  csd n = 64 1.50 -> 1.38 ms, n = 500 14.2 -> 12.6,
+// n = 1024 39.0 -> 35.6, polar n = 2048 40.7 -> 37.8.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... P, class... A>
+void launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  ZCSD_CUDA(cudaLaunchKernelEx(&cfg, kernel, P(args)...));
+}
+#endif
+
 // Optional per-kind kernel timing (CUDA events on the launch stream), used
 // for roofline reports.  prof_begin/prof_end bracket one launch; both are
 // no-ops unless a profiler is active on the calling thread.

@@ -520,6 +520,7 @@ __global__ void __launch_bounds__(1024) chol_inv_kernel(int nb, const T* Zall, i
   const T* Zb = Zall + blockIdx.x * sZ;
   T* N = Nall + blockIdx.x * sN;
   const int i = threadIdx.x >> 5, c = threadIdx.x & 31;
+  chain_wait();
   T m = (i <= c && c < nb) ? Zb[i + (long long)c * ldz] : zero<T>();
   // 1 / x to rounding: FP32 seed, two Newton steps (NaN unless x > 0)
   auto recip = [](double x) {
@@ -547,6 +548,7 @@ __global__ void __launch_bounds__(1024) chol_inv_kernel(int nb, const T* Zall, i
       if (i == j + 1) publish(i);
     }
   }
+  chain_next();
   if (i < nb) {
     const double d = __shfl_sync(0xffffffffu, re(m), i);
     const double s = d > 0.0 ? 1.0 / sqrt(d) : (double)NAN;
@@ -599,7 +601,7 @@ void chol_inv_block(cudaStream_t st, int nb, const T* Z, int ldz, long long sZ, 
                     int batch) {
   if (nb > CHOL_NB) throw CudaFail{cudaErrorInvalidValue, __FILE__, __LINE__};
   ProfToken tok = prof_begin(st);
-  chol_inv_kernel<T><<<batch, 1024, 0, st>>>(nb, Z, ldz, sZ, N, ldn, sN);
+  launch_chained(chol_inv_kernel<T>, dim3(batch), 1024, 0, st, nb, Z, ldz, sZ, N, ldn, sN);
   ZCSD_LAUNCH();
   if (tok.slot >= 0) prof_end(tok, st, PK_POTRF, (2.0 / 3.0) * nb * nb * nb * batch);
 }

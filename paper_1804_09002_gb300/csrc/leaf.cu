@@ -271,6 +271,7 @@ __global__ void __launch_bounds__(THREADS) j32_kernel(LeafDev L, int pass, int s
   __shared__ float nrm[96];
   __shared__ int cmax;
   constexpr int LDS = 128 * NV, NW = THREADS / 32;
+  chain_wait();
   const int l = blockIdx.y, n = L.sz[l];
   const J32Geom g = j32_geom(n, CX, LDS);
   if ((int)blockIdx.x >= g.nblk / 2 || round >= g.nblk - 1) return;
@@ -448,6 +449,7 @@ __global__ void __launch_bounds__(THREADS) j32_kernel(LeafDev L, int pass, int s
     __syncthreads();
     if (worst < J32_STOP * J32_STOP) break;
   }
+  chain_next();
   for (int c = warp; c < 2 * wb; c += NW) {
     const int col = (c < wb ? bp * wb + c : bq * wb + c - wb);
     if (!(col < n && col < (c < wb ? bp + 1 : bq + 1) * wb)) continue;
@@ -823,7 +825,8 @@ void j32_launch(cudaStream_t st, const LeafTable& L, int pass, int sweep, int ro
     return true;
   }();
   (void)attr;
-  j32_kernel<CX, NV, THREADS><<<dim3(ctas, L.nl), THREADS, (size_t)L.maxcols * 128 * NV * 4, st>>>(L, pass, sweep, round);
+  launch_chained(j32_kernel<CX, NV, THREADS>, dim3(ctas, L.nl), THREADS, (size_t)L.maxcols * 128 * NV * 4, st, (const LeafDev&)L,
+                 pass, sweep, round);
   ZCSD_LAUNCH();
 }
 
