@@ -563,10 +563,7 @@ struct ConvSide {
 // Largest exponent of every row of op(X) over all terms and one k segment,
 // |x| < 2^e for the biased exponent E = e + 1022 (INT_MIN: no normal entry), to
 // part[problem][segment][row].  Both operands of a product in one launch
-// (blockIdx.y); eight threads share a row, each with eight loads on their way
-// before the first is used (branches between them, for the weights and the
-// balance, kept one: the 180 MB of a 3001 x 2500 x 4096 product 83 -> 75 us, csd
-// n = 3000 25.8 -> 21.7 ms in this kernel).
+// (blockIdx.y); eight threads share a row.
 __global__ void __launch_bounds__(256) tc_exp_kernel(const __grid_constant__ ConvArgs a0,
                                                      const __grid_constant__ ConvArgs a1, int nsum, int segs, int es,
                                                      const int* ek, int ekpad) {
@@ -587,18 +584,13 @@ __global__ void __launch_bounds__(256) tc_exp_kernel(const __grid_constant__ Con
     for (int j = 0; j < nsum; ++j) {
       const double* X = c.X + j * c.sXj + (i0 + row) * c.si;
       const double w = second ? 1.0 : a0.w.w[j];
-      for (int k = kb; k < ke; k += 64) {
-        double v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = k + 8 * u < ke ? X[(k + 8 * u) * c.sk] : 0.0;
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          if (!c.unit) v[u] *= w;
-          const int E = (__double2hiint(v[u]) >> 20) & 0x7FF;
-          int bal = 0;
-          if (ekb && k + 8 * u < ke && ekb[k + 8 * u] > -2000) bal = c.bsgn * ekb[k + 8 * u];
-          mx = max(mx, E > 0 ? E - 1022 + bal : INT_MIN);
-        }
+#pragma unroll 8
+      for (int k = kb; k < ke; k += 8) {
+        double v = X[k * c.sk];
+        if (!c.unit) v *= w;
+        const int E = (int)((__double_as_longlong(v) >> 52) & 0x7FF);
+        const int bal = ekb ? (ekb[k] > -2000 ? c.bsgn * ekb[k] : 0) : 0;
+        mx = max(mx, E > 0 ? E - 1022 + bal : INT_MIN);
       }
     }
   if (mx != INT_MIN) atomicMax(&rmax[row], mx);
