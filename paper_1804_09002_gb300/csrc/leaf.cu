@@ -64,7 +64,15 @@ constexpr int JAC_THREADS = 256;
 // keep n / 64 SMs busy per leaf with one launch per 32 local rounds; from 257
 // floats per column on 16 columns are faster (twice the SMs, one column per
 // warp and round).  Leaves of at most 96 rows are one pair
-// of blocks: a single CTA, which then runs every sweep in one launch.
+// of blocks: a single CTA, which then runs every sweep in one launch.  Across
+// the blocks a warp keeps j32_owned columns of the first one in registers, so
+// a block has at most j32_cover columns whatever the leaf's size (beside a leaf
+// of 257 floats per column and more, a leaf of 33 to 96 rows has several pairs
+// of 16 columns, which cost nothing next to that leaf's rounds).
+__host__ __device__ constexpr int j32_threads(int lds) { return lds <= 256 ? 1024 : 512; }
+__host__ __device__ constexpr int j32_owned(int lds) { return lds >= 384 ? 1 : 2; }
+__host__ __device__ constexpr int j32_cover(int lds) { return j32_owned(lds) * j32_threads(lds) / 32; }
+
 struct J32Geom {
   int nf;    // floats per column (n, complex 2n)
   int ldg;   // floats per stored column, a multiple of 4
@@ -79,6 +87,7 @@ __host__ __device__ inline J32Geom j32_geom(int n, bool cplx, int lds) {
   const int cap = lds >= 384 ? 16 : 32;
   wmax = wmax > cap ? cap : wmax;
   if (n <= 96 && lds <= 512) wmax = (n + 1) / 2;
+  wmax = wmax > j32_cover(lds) ? j32_cover(lds) : wmax;
   const int half = (n + 2 * wmax - 1) / (2 * wmax);
   g.nblk = 2 * (half < 1 ? 1 : half);
   g.wb = (n + g.nblk - 1) / g.nblk;
@@ -380,8 +389,9 @@ __global__ void __launch_bounds__(THREADS) j32_kernel(LeafDev L, int pass, int s
       }
     }
   };
-  constexpr int KP = LDS >= 384 ? 1 : 2;  // columns of the first block a warp owns across the blocks
-  constexpr bool KEEP = NV <= 8;     // ... in registers
+  static_assert(THREADS == j32_threads(LDS), "the column blocks are sized for these warps");
+  constexpr int KP = j32_owned(LDS);  // columns of the first block a warp owns across the blocks
+  constexpr bool KEEP = NV <= 8;      // ... in registers
   auto cross = [&]() {
     if constexpr (KEEP) {
       float4 x[KP][NV];
@@ -819,7 +829,7 @@ __global__ void leaf_values_kernel(LeafDev L, const T* G, double* lam) {
 
 template <bool CX, int NV>
 void j32_launch(cudaStream_t st, const LeafTable& L, int pass, int sweep, int round, int ctas) {
-  constexpr int THREADS = NV <= 2 ? 1024 : 512;
+  constexpr int THREADS = j32_threads(128 * NV);
   static const bool attr = [] {
     ZCSD_CUDA(cudaFuncSetAttribute(j32_kernel<CX, NV, THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, J32_SMEM));
     return true;
