@@ -60,7 +60,9 @@ typedef struct {
   int zolo_iters;         /* Zolo-pd iterations per polar decomposition (polar(): all passes) */
   int r_terms[4];         /* partial-fraction terms r of each iteration */
   double ell[4];          /* lower end l of [l, 1] entering each iteration */
-  int chol_fallback;      /* always 0 (every Cholesky factorization is positive definite) */
+  int chol_fallback;      /* Zolo-pd iterations redone by Householder QR: 0 for a partial isometry,
+                           * whose Cholesky factorizations are all positive definite; a block of
+                           * norm far above 1 may need it */
   int alg2_used[2];       /* Algorithm 2 applied to block i (2: then the SVD polar fallback) */
   double orth_err[2];     /* ||W_i^* W_i - I||_F of the Zolo-pd factor (polar(): entry 0) */
   double rdiff[2];        /* ||R~_i - R_i||_F / ||R_i||_F (Algorithm 2 check) */

@@ -349,6 +349,20 @@ void shift_terms(cudaStream_t st, int n, const T* X, int ldx, long long sXb, con
 }
 
 template <class T>
+void stack_terms(cudaStream_t st, int n, const T* X, int ldx, long long sXb, const double* sqrtc, int nterms,
+                 T* M, int ldm, long long sM, int batch) {
+  Vec16 s;
+  for (int j = 0; j < MAX_SUM; ++j) s.v[j] = j < nterms ? sqrtc[j] : 0.0;
+  ew2d(st, 2 * n, n, batch * nterms, [=] __device__(int i, int j, int p) {
+    const int bb = p / nterms, jt = p % nterms;
+    T v;
+    if (i < n) v = X[bb * sXb + i + (long long)j * ldx];
+    else v = (i - n == j) ? from_re<T>(s.v[jt]) : zero<T>();
+    M[p * sM + i + (long long)j * ldm] = v;
+  });
+}
+
+template <class T>
 void scale_shift(cudaStream_t st, int n, double alpha, const T* X, int ldx, long long sX, double beta, T* Z, int ldz,
                  long long sZ, int batch) {
   ew2d(st, n, n, batch, [=] __device__(int i, int j, int b) {
@@ -486,9 +500,12 @@ __global__ void diag_real_kernel(int n, const T* X, int ldx, double* d) {
 
 // theta = atan2(S, C) clamped to [0, pi/2], the range of the principal
 // angles (Section 1); rounding can otherwise leave S or C a few ulps below 0.
+// v clamped to [lo, hi]; NaN stays NaN (fmin and fmax would hide a failed factor)
+__device__ inline double clamp_keep_nan(double v, double lo, double hi) { return v <= lo ? lo : (v > hi ? hi : v); }
+
 __global__ void theta_kernel(int n, const double* C, const double* S, double* th) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    th[i] = fmin(fmax(atan2(S[i], C[i]), 0.0), 1.5707963267948966);
+    th[i] = clamp_keep_nan(atan2(S[i], C[i]), 0.0, 1.5707963267948966);
 }
 
 // remark (iv): theta solves sin(theta) - cos(theta) = Lambda, i.e.
@@ -496,8 +513,8 @@ __global__ void theta_kernel(int n, const double* C, const double* S, double* th
 // with Lambda / sqrt(2) clamped to [-1, 1] and theta to [0, pi/2].
 __global__ void theta_lambda_kernel(int n, const double* lam, double* th) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const double x = fmin(fmax(lam[i] * 0.70710678118654752, -1.0), 1.0);
-    th[i] = fmin(fmax(0.78539816339744831 + asin(x), 0.0), 1.5707963267948966);
+    const double x = clamp_keep_nan(lam[i] * 0.70710678118654752, -1.0, 1.0);
+    th[i] = clamp_keep_nan(0.78539816339744831 + asin(x), 0.0, 1.5707963267948966);
   }
 }
 
@@ -649,6 +666,8 @@ void randn(cudaStream_t st, int m, int n, T* X, int ldx, unsigned long long seed
   template void axpby<T>(cudaStream_t, int, int, double, const T*, int, long long, double, T*, int, long long, int); \
   template void sum_parts<T>(cudaStream_t, int, int, T*, int, long long, int, int);                                  \
   template void shift_terms<T>(cudaStream_t, int, const T*, int, long long, const double*, int, T*, int, long long, \
+                               int);                                                                            \
+  template void stack_terms<T>(cudaStream_t, int, const T*, int, long long, const double*, int, T*, int, long long, \
                                int);                                                                            \
   template void scale_shift<T>(cudaStream_t, int, double, const T*, int, long long, double, T*, int, long long, int); \
   template void scale_terms<T>(cudaStream_t, int, int, const double*, int, T*, int, long long, int);            \

@@ -67,6 +67,9 @@ template <class T> void sum_parts(cudaStream_t st, int m, int n, T* X, int ldx, 
 // Y_j = X + shift_j I for j < nterms (shifts on device or by value), Y_j at stride sY
 template <class T> void shift_terms(cudaStream_t st, int n, const T* X, int ldx, long long sXb,
                                     const double* shifts, int nterms, T* Y, int ldy, long long sY, int batch);
+// M_j = [X; sqrt(c_j) I] (2n x n, ld = ldm), for j < nterms of each of `batch` X's
+template <class T> void stack_terms(cudaStream_t st, int n, const T* X, int ldx, long long sXb,
+                                    const double* sqrtc, int nterms, T* M, int ldm, long long sM, int batch);
 // Z_b = alpha X_b + beta I
 template <class T> void scale_shift(cudaStream_t st, int n, double alpha, const T* X, int ldx, long long sX,
                                     double beta, T* Z, int ldz, long long sZ, int batch);

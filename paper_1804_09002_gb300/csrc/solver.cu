@@ -108,8 +108,11 @@ void d2h(Ctx& cx, void* dst, const void* src, size_t bytes) {
 //   * the basis of term j preconditions the terms below it: the columns of
 //     [Q1; sqrt(rho) Q2], rho = c_i / c_j, span [X; sqrt(c_i) I], and their Gram
 //     matrix rho I + (1 - rho) Q1^* Q1 has condition number 1 / rho; its
-//     inverse Cholesky factor orthonormalises them.  It is positive definite
-//     for every X, so there is no pivot to check.
+//     inverse Cholesky factor orthonormalises them.
+// All these Gram matrices are numerically positive definite while n u ||X||_2^2
+// is below the shift 1.8e-7.  Every X here has ||X||_2 <= 1 but for a CSD input
+// that is no partial isometry: a failed factor is NaN, and csd_impl's test of W
+// then takes zolo_householder.
 // Two terms follow from each basis, 1 / rho = 4.7e3 and 2.2e7, so that the
 // chain is four factorizations of two problems long (eight of one leave more
 // SMs idle: a factorization is a chain of 32-column blocks).
@@ -248,6 +251,34 @@ static void zolo_first(cudaStream_t st, Arena& ar, const Plan& pl, int n, int P,
   ar.release(mk);
 }
 
+// An iteration in the form of Section 5, the term X (X^* X + c_j I)^{-1} = Q1
+// Q2^* / sqrt(c_j) by Householder QR of the stacked [X; sqrt(c_j) I] (2n x n,
+// row j of the lower block enters with column j): finite for every finite X.
+template <class T>
+static void zolo_householder(cudaStream_t st, Arena& ar, const Plan& pl, int s, int n, int P, const T* X, T* Xn) {
+  const int r = pl.r[s], m2 = 2 * n;
+  const long long nn = (long long)n * n, sM = 2 * nn;
+  const size_t mk = ar.mark();
+  T* M = ar.get<T>(sM * P * r);
+  T* E = ar.get<T>(sM * P * r);
+  stack_terms<T>(st, n, X, n, nn, pl.sqrtc[s], r, M, m2, sM, P);
+  QRStore<T> q = qr_alloc<T>(ar, m2, n, n + 1, P * r);
+  qr_factor<T>(st, ar, q, M, m2, sM);
+  qr_form_q<T>(st, ar, q, E, m2, sM);
+  GemmArgs<T> g;  // X_new = mhat X + sum_j w_j Q1_j Q2_j^* (Q2 upper triangular)
+  g.batch = P;
+  g.m = n; g.n = n; g.k = n; g.opA = OP_N; g.opB = OP_C; g.kflags = K_FROM_COL;
+  g.A = E; g.lda = m2; g.sA = sM * r; g.sAj = sM;
+  g.B = E + n; g.ldb = m2; g.sB = sM * r; g.sBj = sM;
+  g.nsum = r;
+  for (int j = 0; j < r; ++j) g.w[j] = pl.w[s][j];
+  g.Cin = X; g.ldcin = n; g.sCin = nn;
+  g.C = Xn; g.ldc = n; g.sC = nn;
+  g.alpha = from_re<T>(1.0); g.beta = from_re<T>(pl.mhat[s]); g.site = GS_ZOLO_COMBINE;
+  gemm_terms(g, st);
+  ar.release(mk);
+}
+
 // Later iterations, Cholesky form: X_new = mhat (X + X sum_j a_j Z_j^{-1}),
 // Z_j = X^* X + c_j I = R_j^* R_j.  X's singular values lie in [l_s, 1], so the
 // Z_j are well conditioned and their inverses N_j N_j^*, N_j = R_j^{-1}, are
@@ -303,7 +334,8 @@ static void zolo_next(cudaStream_t st, Arena& ar, const Plan& pl, int s, int n, 
 // X_{k+1} = M (X_k + sum_j a_j X_k (X_k^* X_k + c_{2j-1} I)^{-1}); the first
 // iteration from orthonormal bases, later ones in Cholesky form.
 template <class T>
-void zolo_pd(Ctx& cx, Arena& ar, int n, int P, const T* X0, T* W, PolarDiag* pd, int stop_after, int reduced_slices) {
+void zolo_pd(Ctx& cx, Arena& ar, int n, int P, const T* X0, T* W, PolarDiag* pd, int stop_after, int reduced_slices,
+             bool householder) {
   cudaStream_t st = cx.stream;
   const Plan& pl = get_plan(cx);
   const int steps = (stop_after > 0) ? std::min(stop_after, pl.steps) : pl.steps;
@@ -318,7 +350,9 @@ void zolo_pd(Ctx& cx, Arena& ar, int n, int P, const T* X0, T* W, PolarDiag* pd,
     // X is well conditioned after the first iteration; with reduced_slices its
     // Gram product and the products with the inverses then keep fewer bits of
     // their operands, the Cholesky factorizations themselves do not.
-    if (s == 0) {
+    if (householder) {
+      zolo_householder<T>(st, ar, pl, s, n, P, X, Xn);
+    } else if (s == 0) {
       zolo_first<T>(st, ar, pl, n, P, X, Xn);
     } else {
       const bool fewer = reduced_slices == 5 || reduced_slices == 6;
@@ -332,8 +366,8 @@ void zolo_pd(Ctx& cx, Arena& ar, int n, int P, const T* X0, T* W, PolarDiag* pd,
   ar.release(mk);
 }
 
-template void zolo_pd<double>(Ctx&, Arena&, int, int, const double*, double*, PolarDiag*, int, int);
-template void zolo_pd<z64>(Ctx&, Arena&, int, int, const z64*, z64*, PolarDiag*, int, int);
+template void zolo_pd<double>(Ctx&, Arena&, int, int, const double*, double*, PolarDiag*, int, int, bool);
+template void zolo_pd<z64>(Ctx&, Arena&, int, int, const z64*, z64*, PolarDiag*, int, int, bool);
 
 // ---------------------------------------------------------------- CSD
 template <class T>
@@ -361,8 +395,7 @@ int csd_impl(Ctx& cx, Arena& ar, int n, const T* A1, int lda1, const T* A2, int 
   d2h(cx, cx.hs.d, sc, 3 * sizeof(double));
   if (cx.hs.d[0] != 0.0) return CSD_ERR_NONFINITE;
   const double fro = cx.hs.d[1] + cx.hs.d[2];
-  int r = (int)std::floor(fro + 0.5);
-  r = std::max(0, std::min(n, r));
+  const int r = fro >= n ? n : (int)std::floor(fro + 0.5);
   const double mu = (r == n) ? 0.0 : 2.0;
   if (info) {
     info->rank = r;
@@ -373,11 +406,13 @@ int csd_impl(Ctx& cx, Arena& ar, int n, const T* A1, int lda1, const T* A2, int 
       info->ell[s] = s < pl.steps ? pl.ell[s] : 0.0;
     }
   }
-  // ---- lines 1-2: W_i H_i = A_i (both polar decompositions in one batch)
+  // ---- lines 1-2: W_i H_i = A_i (both polar decompositions in one batch),
+  // and the orthogonality of W_i
   PolarDiag pd;
-  zolo_pd<T>(cx, ar, n, 2, Apk, W, &pd, 0, (cx.mixed_scope & 1u) ? cx.mixed_slices : 0);
   const T one = from_re<T>(1.0), zer = zero<T>();
-  {
+  double orth[2];
+  for (int redo = 0; redo < 2; ++redo) {
+    zolo_pd<T>(cx, ar, n, 2, Apk, W, &pd, 0, (cx.mixed_scope & 1u) ? cx.mixed_slices : 0, redo != 0);
     GemmArgs<T> g;  // H_i = sym(W_i^* A_i)
     g.batch = 2;
     g.m = n; g.n = n; g.k = n; g.opA = OP_C; g.opB = OP_N;
@@ -388,25 +423,20 @@ int csd_impl(Ctx& cx, Arena& ar, int n, const T* A1, int lda1, const T* A2, int 
     g.site = GS_H;
     gemm(g, st);
     symmetrize<T>(st, n, H, n, nn, H, n, nn, 2);
-  }
-  // ---- orthogonality of W_i; Algorithm 2 where W_i is not orthonormal
-  {
     const size_t mk = ar.mark();
     T* Gw = ar.get<T>(2 * nn);
-    GemmArgs<T> g;
-    g.batch = 2;
-    g.m = n; g.n = n; g.k = n; g.opA = OP_C; g.opB = OP_N;
-    g.A = W; g.lda = n; g.sA = nn;
-    g.B = W; g.ldb = n; g.sB = nn;
-    g.C = Gw; g.ldc = n; g.sC = nn;
-    g.alpha = one; g.beta = zer;
+    g.B = W;
+    g.C = Gw;
     g.site = GS_ORTH;
     gemm(g, st);
     fro2<T>(st, n, n, Gw, n, nn, 1.0, sc + 4, 2, scratch);
     d2h(cx, cx.hs.d, sc + 4, 2 * sizeof(double));
     ar.release(mk);
+    for (int i = 0; i < 2; ++i) orth[i] = std::sqrt(cx.hs.d[i]);
+    if (info) info->chol_fallback = redo * pl.steps;
+    // a Cholesky factor that failed (blocks of a norm far above 1) leaves NaN
+    if (std::isfinite(orth[0]) && std::isfinite(orth[1])) break;
   }
-  const double orth[2] = {std::sqrt(cx.hs.d[0]), std::sqrt(cx.hs.d[1])};
   int status = CSD_OK;
   if (info) {
     info->orth_err[0] = orth[0];
@@ -449,9 +479,9 @@ int csd_impl(Ctx& cx, Arena& ar, int n, const T* A1, int lda1, const T* A2, int 
     const double rd = std::sqrt(cx.hs.d[0]) / std::max(std::sqrt(fro / 2.0), 1e-300);
     if (info) { info->alg2_used[i] = 1; info->rdiff[i] = rd; }
     ar.release(mk);
-    if (rd > 1e3 * n * U_ROUND || (cx.alg2_svd_factor >= 0.0 && rd >= cx.alg2_svd_factor * n * U_ROUND)) {
+    if (!(rd <= 1e3 * n * U_ROUND) || (cx.alg2_svd_factor >= 0.0 && rd >= cx.alg2_svd_factor * n * U_ROUND)) {
       if (cx.alg2_svd_factor < 0.0) {
-        status = CSD_WARN_ALG2_RCHECK;
+        if (status != CSD_ERR_NOT_CONVERGED) status = std::isfinite(rd) ? CSD_WARN_ALG2_RCHECK : CSD_ERR_NOT_CONVERGED;
       } else {
         // Section 5.1: ||R~ - R|| not O(u), so W_i H_i is not a backward
         // stable polar decomposition of A_i; take the polar decomposition
@@ -463,10 +493,11 @@ int csd_impl(Ctx& cx, Arena& ar, int n, const T* A1, int lda1, const T* A2, int 
       }
     }
   };
-  // full rank: Algorithm 2 where W_i is not orthonormal
+  // full rank: Algorithm 2 where W_i is not orthonormal; at any rank where it
+  // is not finite
   const double orth_tol = 50.0 * n * U_ROUND;
-  for (int i = 0; i < 2 && mu == 0.0; ++i)
-    if (orth[i] > orth_tol) alg2(i);
+  for (int i = 0; i < 2; ++i)
+    if (mu == 0.0 ? !(orth[i] <= orth_tol) : !std::isfinite(orth[i])) alg2(i);
   // ---- line 4: B = H2 - H1 + mu (I - A^* A)
   {
     const size_t mk = ar.mark();

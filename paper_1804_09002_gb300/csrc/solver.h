@@ -88,11 +88,13 @@ struct ReducedScope {
 // stop_after > 0 stops after that many iterations (the iterate X_k).
 // reduced_slices = 5 or 6 runs the Gram product and the products with the
 // inverses of the Cholesky-form iterations with 45 or 51 bits of the operands
-// (tensor-core path).  No device-to-host read, so the call can be captured in
-// a CUDA graph.
+// (tensor-core path).  householder: every iteration by Householder QR of the
+// stacked [X; sqrt(c) I], for an X0 whose Cholesky factors fail (||X0||_2 far
+// above 1; NaN in W then).  No device-to-host read, so the call can be captured
+// in a CUDA graph.
 template <class T>
 void zolo_pd(Ctx& cx, Arena& ar, int n, int P, const T* X0, T* W, PolarDiag* pd, int stop_after = 0,
-             int reduced_slices = 0);
+             int reduced_slices = 0, bool householder = false);
 
 // Counters of one Zolo-eig call.
 struct EigDiag {
