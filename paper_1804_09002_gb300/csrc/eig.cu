@@ -458,7 +458,14 @@ void heig_impl(Ctx& cx, Arena& ar, int n, const T* Bin, int ldb, double* lam, T*
         // orthogonal to rounding, so the factor only has their own condition
         // numbers, of order k^2; two steps of Q <- Q - Q E / 2, E = Q^* Q - I of
         // order k^2 u, restore orthonormality.  (Householder QR of P Omega took a
-        // fifth of a split, a chain of n / 32 panels.)  Q1 inherits an error of
+        // fifth of a split, a chain of n / 32 panels.)  A draw of Omega some
+        // hundred times worse than that leaves more: the first step squares E,
+        // the second keeps E1 to 24 bits and squares it again, so the basis is
+        // orthonormal to rounding while ||E1||_F <= 2^-29.  A block beyond that
+        // (or NaN: the Gram matrix was not positive definite) is not tested but
+        // goes through the pass again with Householder QR of P Omega, Omega a
+        // new draw, which is orthonormal for any draw.
+        // Q1 inherits an error of
         // order k u from the condition of P Omega; a block whose split fails
         // the off-block test gets one step of subspace iteration from Q, whose
         // P Q1 ~ Q1 are well conditioned, before a new shift (and a new polar
@@ -466,8 +473,9 @@ void heig_impl(Ctx& cx, Arena& ar, int n, const T* Bin, int ldb, double* lam, T*
         T* Pm = ar.get<T>(nbb * Pa);
         blk_proj_pad<T><<<dim3(ew_grid(nbb), Pa), 256, 0, st>>>(Wm, nb, dsz, Pm);
         ZCSD_LAUNCH();
-        randn<T>(st, nb, nb * Pa, Om, nb,
-                 cx.seed + 7919ull * (unsigned long long)(depth * 4096 + attempt * 256 + (int)gi) + 1ull);
+        const unsigned long long seed =
+            cx.seed + 7919ull * (unsigned long long)(depth * 4096 + attempt * 256 + (int)gi) + 1ull;
+        randn<T>(st, nb, nb * Pa, Om, nb, seed);
         auto bgemm = [&](int opA, const T* A, const T* Bp, T* C) {
           GemmArgs<T> g;
           g.batch = Pa;
@@ -484,48 +492,58 @@ void heig_impl(Ctx& cx, Arena& ar, int n, const T* Bin, int ldb, double* lam, T*
           if (k[a] >= 0) cand.push_back(a);
         const int* dk = upload(ar, st, k);
         T* Nf = ar.get<T>(nbb * Pa);
-        for (int pass = 0; pass < 2 && !cand.empty(); ++pass) {
-          T* basis = pass == 0 ? Om : Qf;
+        bool householder = false;  // the pass again, after a bad draw
+        for (int pass = 0; pass < 2 && !cand.empty();) {
+          if (householder) randn<T>(st, nb, nb * Pa, Om, nb, seed + (1ull << 48));
+          T* basis = pass == 0 || householder ? Om : Qf;
           bgemm(OP_N, Pm, basis, Wm);  // P Omega, then P Q
-          blk_two_bases<T><<<dim3(ew_grid(nbb), Pa), 256, 0, st>>>(Wm, basis, nb, dsz, dk, Tm);
-          ZCSD_LAUNCH();
-          auto gram = [&](const T* A) {  // Wm = A^* A (upper triangle)
-            GemmArgs<T> g;
-            g.batch = Pa;
-            g.m = nb; g.n = nb; g.k = nb; g.opA = OP_C; g.opB = OP_N; g.uplo = 1;
-            g.A = A; g.lda = nb; g.sA = nbb;
-            g.B = A; g.ldb = nb; g.sB = nbb;
-            g.C = Wm; g.ldc = nb; g.sC = nbb;
-            g.alpha = one; g.beta = zer; g.site = GS_EIG;
-            gemm(g, st);
-          };
-          gram(Tm);
-          ZCSD_CUDA(cudaMemsetAsync(Nf, 0, sizeof(T) * nbb * Pa, st));
-          chol_inverse<T>(st, ar, nb, Wm, nb, nbb, Nf, nb, nbb, Pa);
-          {
-            GemmArgs<T> g;  // Q = Y N
-            g.batch = Pa;
-            g.m = nb; g.n = nb; g.k = nb; g.opA = OP_N; g.opB = OP_N; g.kflags = K_TO_COL;
-            g.A = Tm; g.lda = nb; g.sA = nbb;
-            g.B = Nf; g.ldb = nb; g.sB = nbb;
-            g.C = Qf; g.ldc = nb; g.sC = nbb;
-            g.alpha = one; g.beta = zer; g.site = GS_EIG;
-            gemm(g, st);
-          }
-          for (int it = 0; it < 2; ++it) {  // Q <- Q - Q E / 2
-            T* from = it == 0 ? Qf : Tm;
-            gram(from);
-            minus_eye<T>(st, nb, Wm, nb, nbb, Nf, nb, nbb, Pa);
-            ReducedScope scope(1u << GS_ZOLO_POLISH, it == 0 ? 45 : 24);
-            GemmArgs<T> g;
-            g.batch = Pa;
-            g.m = nb; g.n = nb; g.k = nb; g.opA = OP_N; g.opB = OP_N;
-            g.A = from; g.lda = nb; g.sA = nbb;
-            g.B = Nf; g.ldb = nb; g.sB = nbb;
-            g.Cin = from; g.ldcin = nb; g.sCin = nbb;
-            g.C = it == 0 ? Tm : Qf; g.ldc = nb; g.sC = nbb;
-            g.alpha = from_re<T>(-0.5); g.beta = one; g.site = GS_ZOLO_POLISH;
-            gemm(g, st);
+          if (householder) {
+            const size_t mq = ar.mark();
+            QRStore<T> q = qr_alloc<T>(ar, nb, nb, nb, Pa);
+            qr_factor<T>(st, ar, q, Wm, nb, nbb);
+            qr_form_q<T>(st, ar, q, Qf, nb, nbb);
+            ar.release(mq);
+          } else {
+            blk_two_bases<T><<<dim3(ew_grid(nbb), Pa), 256, 0, st>>>(Wm, basis, nb, dsz, dk, Tm);
+            ZCSD_LAUNCH();
+            auto gram = [&](const T* A) {  // Wm = A^* A (upper triangle)
+              GemmArgs<T> g;
+              g.batch = Pa;
+              g.m = nb; g.n = nb; g.k = nb; g.opA = OP_C; g.opB = OP_N; g.uplo = 1;
+              g.A = A; g.lda = nb; g.sA = nbb;
+              g.B = A; g.ldb = nb; g.sB = nbb;
+              g.C = Wm; g.ldc = nb; g.sC = nbb;
+              g.alpha = one; g.beta = zer; g.site = GS_EIG;
+              gemm(g, st);
+            };
+            gram(Tm);
+            ZCSD_CUDA(cudaMemsetAsync(Nf, 0, sizeof(T) * nbb * Pa, st));
+            chol_inverse<T>(st, ar, nb, Wm, nb, nbb, Nf, nb, nbb, Pa);
+            {
+              GemmArgs<T> g;  // Q = Y N
+              g.batch = Pa;
+              g.m = nb; g.n = nb; g.k = nb; g.opA = OP_N; g.opB = OP_N; g.kflags = K_TO_COL;
+              g.A = Tm; g.lda = nb; g.sA = nbb;
+              g.B = Nf; g.ldb = nb; g.sB = nbb;
+              g.C = Qf; g.ldc = nb; g.sC = nbb;
+              g.alpha = one; g.beta = zer; g.site = GS_EIG;
+              gemm(g, st);
+            }
+            for (int it = 0; it < 2; ++it) {  // Q <- Q - Q E / 2
+              T* from = it == 0 ? Qf : Tm;
+              gram(from);
+              minus_eye<T>(st, nb, Wm, nb, nbb, Nf, nb, nbb, Pa);
+              ReducedScope scope(1u << GS_ZOLO_POLISH, it == 0 ? 45 : 24);
+              GemmArgs<T> g;
+              g.batch = Pa;
+              g.m = nb; g.n = nb; g.k = nb; g.opA = OP_N; g.opB = OP_N;
+              g.A = from; g.lda = nb; g.sA = nbb;
+              g.B = Nf; g.ldb = nb; g.sB = nbb;
+              g.Cin = from; g.ldcin = nb; g.sCin = nbb;
+              g.C = it == 0 ? Tm : Qf; g.ldc = nb; g.sC = nbb;
+              g.alpha = from_re<T>(-0.5); g.beta = one; g.site = GS_ZOLO_POLISH;
+              gemm(g, st);
+            }
           }
           // ---- B' = Q^* B_sub Q = ||B_sub - sI||_F Q^* X Q + s I: the shift
           // is added back exactly, so the departure of Q from orthogonality
@@ -533,18 +551,21 @@ void heig_impl(Ctx& cx, Arena& ar, int n, const T* Bin, int ldb, double* lam, T*
           // off-diagonal block
           bgemm(OP_N, X, Qf, Tm);
           bgemm(OP_C, Qf, Tm, Om);
-          std::vector<long long> boff;
+          std::vector<long long> boff, eoff;
           std::vector<int> rm, rc;
           for (int a : cand) {
             boff.push_back((long long)a * nbb + k[a]);
             rm.push_back(sz[a] - k[a]);
             rc.push_back(k[a]);
+            eoff.push_back((long long)a * nbb);
           }
-          double* doffa = ar.get<double>(cand.size());
+          double* doffa = ar.get<double>(2 * cand.size());
           blk_fro2<T>(st, ar, Om, nb, boff, rm, rc, nullptr, doffa);
-          const std::vector<double> h = download(cx, doffa, cand.size());
+          const std::vector<int> whole(cand.size(), nb);
+          if (!householder) blk_fro2<T>(st, ar, Nf, nb, eoff, whole, whole, nullptr, doffa + cand.size());  // E1
+          const std::vector<double> h = download(cx, doffa, (householder ? 1 : 2) * cand.size());
           std::vector<int> accept(Pa, 0), retry;
-          bool any_acc = false;
+          bool any_acc = false, redo = false;
           for (size_t i = 0; i < cand.size(); ++i) {
             const int a = cand[i];
             SplitState& w = work[grp[a]];
@@ -553,6 +574,11 @@ void heig_impl(Ctx& cx, Arena& ar, int n, const T* Bin, int ldb, double* lam, T*
               fprintf(stderr, "zolo-eig:   off=%d pass=%d k=%d ||B21||=%.3e tol=%.3e\n", w.b.off, pass, k[a], offa,
                       w.off_tol);
             if (cx.test_flags & TEST_REJECT_EIG_SPLITS) continue;  // injected failure (tests only)
+            if (!householder && !(h[cand.size() + i] <= 0x1p-58)) {
+              retry.push_back(a);
+              redo = true;
+              continue;
+            }
             if (!(offa <= w.off_tol)) {
               retry.push_back(a);
               continue;
@@ -584,6 +610,8 @@ void heig_impl(Ctx& cx, Arena& ar, int n, const T* Bin, int ldb, double* lam, T*
             }
           }
           cand.swap(retry);
+          householder = redo;
+          if (!redo) ++pass;
         }
         if (debug) {
           ZCSD_CUDA(cudaStreamSynchronize(st));
