@@ -175,7 +175,9 @@ __global__ void __launch_bounds__(NT, 2) gemm_kernel(GemmArgs<T> g) {
 // The products between the 32-column blocks of an inverse Cholesky factor fill
 // the chip with 8 x 8 tiles only (csd n = 64 1.65 -> 1.53 ms, n = 201 6.60 ->
 // 6.13, polar n = 2048 42.8 -> 41.1, together with what the kernel leaves out).
-// A product in place needs one tile over the whole of what it overwrites.
+// A product in place needs one tile over the whole of what it overwrites, and
+// the column tiles must fit a grid's second dimension (more than 524 280 columns
+// are too many for 8-column tiles).
 enum GemmTile { TILE_64 = 0, TILE_32x128, TILE_32, TILE_16, TILE_16x8, TILE_8, TILES };
 constexpr int TILE_M[TILES] = {64, 32, 32, 16, 16, 8}, TILE_N[TILES] = {64, 128, 32, 16, 8, 8};
 
@@ -185,6 +187,7 @@ int pick_tile(const GemmArgs<T>& g) {
   double cost = 0.0;
   for (int t = 0; t < TILES; ++t) {
     if ((g.C == g.B && TILE_M[t] < g.m) || (g.C == g.A && TILE_N[t] < g.n)) continue;
+    if (ceil_div(g.n, TILE_N[t]) > 65535) continue;
     const long long tm = ceil_div(g.m, TILE_M[t]), tn = ceil_div(g.n, TILE_N[t]);
     long long tiles = tm * tn;
     if (g.uplo) tiles = (tiles + std::min(tm, tn)) / 2;
