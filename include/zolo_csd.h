@@ -382,9 +382,13 @@ int csd_fp64_peak(int device, int kind, double* tflops, double* ms);
  * data, runs once outside a capture, then captures the whole batch into a
  * CUDA graph; later runs on the same buffers only launch the graph (new
  * buffers are captured again).  status (host, count ints, may be NULL)
- * receives 0, CSD_ERR_NOT_CONVERGED or CSD_ERR_INTERNAL per instance.  The plan owns its device
- * workspace (grown on demand) and uses the context's stream; destroy the
- * plan before the context.
+ * receives 0, CSD_ERR_NOT_CONVERGED or CSD_ERR_INTERNAL per instance.
+ * The plan owns its device workspace (grown on demand): buckets run side by
+ * side on up to eight streams, each with the workspace of its largest bucket,
+ * as long as these together take no more than 48 GiB and a quarter of the
+ * memory that is free at the plan's first run; one stream's workspace is
+ * allocated in any case.  It uses the context's stream; destroy the plan
+ * before the context.
  * create returns 0, -1 (NULL context), -2 (count < 1), -3 (bad sizes),
  * -4 (NULL plan pointer) or CSD_ERR_ALLOC; run returns 0, -k, or a
  * CSD_ERR_* code. */

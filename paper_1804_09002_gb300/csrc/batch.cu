@@ -42,7 +42,11 @@ namespace {
 
 constexpr int BATCH_MAX_N = 1024;
 constexpr int MAX_LANES = 8;
-constexpr size_t LANE_BYTES = (size_t)48 << 30;  // workspace of all lanes together, where more than one needs it
+// Workspace of all lanes together, where more than one needs it: at most this
+// much and a quarter of the memory that is free when the plan lays out its
+// buckets, so that the caller's later allocations meet the larger part of it.
+constexpr size_t LANE_BYTES = (size_t)48 << 30;
+constexpr int LANE_FREE_PARTS = 4;
 constexpr int BATCH_SWEEPS = 30;  // FP64 Jacobi sweeps at most of a leaf that the refinement leaves open
 
 struct Bucket {
@@ -295,8 +299,10 @@ int build_buckets(csd_batch* b, int gran) {
   b->persist_bytes = (pbytes + 255) & ~(size_t)255;
   // lanes: the largest buckets first, each to the lane with the least work so
   // far (a bucket's time grows with its size, hardly with its instances); as
-  // many lanes as fit LANE_BYTES and the memory that is free (one lane needs no
-  // more than the largest bucket)
+  // many lanes as fit the limit (one lane needs no more than the largest bucket)
+  size_t free_bytes = 0, device_bytes = 0;
+  if (cudaMemGetInfo(&free_bytes, &device_bytes) != cudaSuccess) cudaGetLastError();
+  const size_t limit = std::min(LANE_BYTES, free_bytes / LANE_FREE_PARTS);
   std::vector<int> order((int)b->buckets.size());
   for (size_t k = 0; k < order.size(); ++k) order[k] = (int)k;
   std::sort(order.begin(), order.end(), [&](int x, int y) { return b->buckets[x].nb > b->buckets[y].nb; });
@@ -314,7 +320,7 @@ int build_buckets(csd_batch* b, int gran) {
       total += bytes[l];
     }
     b->lane_off[b->lanes] = total;
-    if (b->lanes > 1 && total > LANE_BYTES) continue;
+    if (b->lanes > 1 && total > limit) continue;
     b->ws_bytes = b->persist_bytes + total;
     if (cudaMalloc((void**)&b->ws, b->ws_bytes) == cudaSuccess) break;
     cudaGetLastError();
