@@ -13,11 +13,14 @@
 //     Appl. Math. 35, 2018): S = X^* B X, P = X^* X, lambda_j = s_jj / p_jj,
 //     E_ij = (s_ij - lambda_j p_ij) / (lambda_j - lambda_i), X <- X + X E.
 //     Each step squares the error and is three products; a pair closer than
-//     the coupling of its columns is only re-orthogonalised.
+//     four times the coupling of its columns is only re-orthogonalised.
 //     Leaves that end with such clusters repeat stages 1 and 2 on them: every
 //     cluster's block of S, shifted and scaled by itself, is a new FP32
 //     problem at the same place (blocks of different clusters have exactly
-//     orthogonal columns, so one solve serves all).
+//     orthogonal columns, so one solve serves all).  A pass resolves gaps about
+//     1e-3 of its clusters' width, so spectra graded over FP64's range (small
+//     angles) take up to six (n = 1000, lambda = 2^(-40 i / n): 65 ms; left to
+//     stage 3 after three passes, 8.0 s).
 //  3. Leaves that still hold an off-diagonal entry above rounding level are
 //     finished by FP64 two-sided Jacobi on S, a cluster of CTAs per leaf, one
 //     launch (on B itself, should X not be orthonormal).
@@ -52,7 +55,9 @@ constexpr int PRE_PARTS = 32, POW_STEPS = 7;
 constexpr int J32_SMEM = 200 * 1024;    // columns of a block pair
 constexpr int REF_STEPS = 7;            // refinement steps of a pass at most, ...
 constexpr int ORTHO_STEPS = 2;          // ... the last of them only re-orthogonalise
-constexpr int PASSES = 3;               // passes of stages 1 and 2 (later ones on clusters)
+constexpr int PASSES = 8;               // passes of stages 1 and 2 (later ones on clusters), ...
+constexpr int PASSES_FIXED = 2;         // ... of a call without reads, where each is launched in any case
+constexpr double GAP = 4.0;             // pairs closer than this many couplings are not rotated but clustered
 constexpr int OFF_N = PASSES * (REF_STEPS + 1);  // looks at a leaf's state
 constexpr unsigned LEAF_OPEN = 1, LEAF_SKEW = 2;  // off-diagonal above rounding; X not orthonormal
 constexpr int LEAF_TC = 384;            // rows from which tensor-core products pay
@@ -578,7 +583,9 @@ __global__ void __launch_bounds__(MM_R * MM_C) leaf_mm_kernel(LeafDev L, int it,
 
 // Column j of a leaf (a warp): lambda_j, rho_j = ||(s_ij - lambda_j p_ij)_{i != j}||
 // and the leaf's state at look `it`: 0 when every coupling and |p_ij - delta_ij|
-// is at its rounding level.
+// is at its rounding level.  A pass that ends with couplings of u ||B||_F at most
+// ends the leaf as well: the FP64 stage would not rotate them, and a wide leaf's
+// rounding can keep a cluster's couplings just above the other level for ever.
 template <class T>
 __global__ void leaf_state_kernel(LeafDev L, int it, const T* S, const T* P) {
   const int l = blockIdx.y, n = L.sz[l], lane = threadIdx.x & 31;
@@ -586,7 +593,8 @@ __global__ void leaf_state_kernel(LeafDev L, int it, const T* S, const T* P) {
   if (j >= n || leaf_ended(L, l, it - 1)) return;
   const T* s = S + L.goff[l] + (long long)j * n;
   const T* p = P + L.goff[l] + (long long)j * n;
-  const double tolS = off_tol(L, l), tolP = 24.0 * 0x1p-53;
+  const bool last = it % (REF_STEPS + 1) == REF_STEPS;
+  const double tolS = last ? fmax(off_tol(L, l), 0x1p-53 * L.c[l]) : off_tol(L, l), tolP = 24.0 * 0x1p-53;
   const double pjj = re(p[j]), lj = pjj > 0.0 ? re(s[j]) / pjj : 0.0;
   double rho = 0.0;
   unsigned flag = 0;
@@ -611,9 +619,10 @@ __global__ void leaf_state_kernel(LeafDev L, int it, const T* S, const T* P) {
 }
 
 // The correction E.  A pair is rotated when its eigenvalues are further apart
-// than twice the coupling of either column (then the rows of E have norm at
-// most 1/2, and the step converges quadratically) and its coupling is above
-// rounding; the others are only re-orthogonalised.
+// than GAP times the coupling of either column (then the rows of E have norm at
+// most 1/4, X stays within some per cent of orthonormal and the step converges
+// quadratically; with twice the coupling graded spectra lost orthonormality)
+// and its coupling is above rounding; the others are only re-orthogonalised.
 template <class T>
 __global__ void leaf_correction_kernel(LeafDev L, int it, int ortho_only, const T* S, const T* P, T* E) {
   const int l = blockIdx.y, n = L.sz[l];
@@ -631,7 +640,7 @@ __global__ void leaf_correction_kernel(LeafDev L, int it, int ortho_only, const 
       // e_ij + conj(e_ji) = -p_ij: both entries of a pair take the same branch
       const T num = sub(S[o + e], scal(lam[j], p)), mirror = sub(S[o + e], scal(lam[i], p));
       const double den = lam[j] - lam[i];
-      if (!ortho_only && fmax(abs2(num), abs2(mirror)) > tol * tol && fabs(den) > 2.0 * fmax(rho[i], rho[j])) v = scal(1.0 / den, num);
+      if (!ortho_only && fmax(abs2(num), abs2(mirror)) > tol * tol && fabs(den) > GAP * fmax(rho[i], rho[j])) v = scal(1.0 / den, num);
       else v = scal(-0.5, p);
     }
     E[o + e] = v;
@@ -639,11 +648,14 @@ __global__ void leaf_correction_kernel(LeafDev L, int it, int ortho_only, const 
 }
 
 // Next pass of stage 1, one CTA per open leaf: the columns in ascending order
-// of lambda fall into clusters where neighbours are closer than twice their
-// coupling; cluster k's shift (its mean lambda), scale (1 / Frobenius norm of
+// of lambda fall into clusters, cut where every column below is GAP couplings
+// away from every column above, so that each pair which the refinement does not
+// rotate is inside a cluster (a cut between neighbours that are far apart by
+// their own couplings alone leaves pairs which nothing treats, and the passes
+// stall); cluster k's shift (its mean lambda), scale (1 / Frobenius norm of
 // its shifted block, from lambda and rho) and label.
 __global__ void __launch_bounds__(1024) leaf_cluster_kernel(LeafDev L, int pass) {
-  __shared__ double sl[LEAF_MAX], sr[LEAF_MAX];
+  __shared__ double sl[LEAF_MAX], sr[LEAF_MAX], below[LEAF_MAX];
   __shared__ int start[LEAF_MAX];
   const int l = blockIdx.x, n = L.sz[l], tid = threadIdx.x;
   if (leaf_ended(L, l, pass * (REF_STEPS + 1) - 1)) return;
@@ -660,9 +672,13 @@ __global__ void __launch_bounds__(1024) leaf_cluster_kernel(LeafDev L, int pass)
   }
   __syncthreads();
   if (tid == 0) {
+    double lowest = INFINITY;  // of lambda - GAP rho over the columns from k on
+    for (int k = n - 1; k >= 0; --k) below[k] = lowest = fmin(lowest, sl[k] - GAP * sr[k]);
+    double highest = -INFINITY;  // of lambda + GAP rho over the columns before k
     int s0 = 0;
     for (int k = 0; k < n; ++k) {
-      if (k > 0 && sl[k] - sl[k - 1] > 2.0 * fmax(sr[k], sr[k - 1])) s0 = k;
+      if (k > 0 && sl[k] > highest && below[k] > sl[k - 1]) s0 = k;
+      highest = fmax(highest, sl[k] + GAP * sr[k]);
       start[k] = s0;
     }
   }
@@ -813,10 +829,10 @@ __global__ void __cluster_dims__(JAC_CTAS, 1, 1) __launch_bounds__(JAC_THREADS)
   if (rank == 0 && tid == 0) L.done[l] = conv ? 1 : 0;
 }
 
-// the last look of a call with two passes becomes the last of all
+// the last look of a call with PASSES_FIXED passes becomes the last of all
 __global__ void leaf_last_kernel(LeafDev L) {
   const int l = blockIdx.x * blockDim.x + threadIdx.x;
-  if (l < L.nl) L.off[l * OFF_N + OFF_N - 1] = L.off[l * OFF_N + 2 * (REF_STEPS + 1) - 1];
+  if (l < L.nl) L.off[l * OFF_N + OFF_N - 1] = L.off[l * OFF_N + PASSES_FIXED * (REF_STEPS + 1) - 1];
 }
 
 // lambda[loff_l + j] = s_jj (blockIdx.y = leaf)
@@ -964,7 +980,10 @@ void leaf_solve(Ctx& cx, Arena& ar, const LeafTable& L, const T* B, double* lam,
     }
   };
   bool any = true;
-  for (int pass = 0; pass < (sync_free ? 2 : PASSES) && any; ++pass) {
+  const int passes = sync_free ? PASSES_FIXED : PASSES;
+  for (int pass = 0; pass < passes && any; ++pass) {
+    // two steps more of the kind at the end: stage 3 starts from S only where X is orthonormal
+    const int ortho = pass + 1 < passes ? ORTHO_STEPS : 2 * ORTHO_STEPS;
     const int look0 = pass * (REF_STEPS + 1);
     if (pass > 0) {
       leaf_cluster_kernel<<<L.nl, 1024, 0, st>>>(L, pass);
@@ -1010,7 +1029,7 @@ void leaf_solve(Ctx& cx, Arena& ar, const LeafTable& L, const T* B, double* lam,
       // stop once every leaf has ended (rarely before the third look)
       if (!sync_free && (it >= 2 || !big.empty()) && !(any = read_state(look))) break;
       if (it == REF_STEPS) break;
-      leaf_correction_kernel<T><<<dim3(ew, L.nl), 256, 0, st>>>(L, look, it >= REF_STEPS - ORTHO_STEPS, S, P, Tm);
+      leaf_correction_kernel<T><<<dim3(ew, L.nl), 256, 0, st>>>(L, look, it >= REF_STEPS - ortho, S, P, Tm);
       ZCSD_LAUNCH();
       leaf_mm_kernel<T, MM_XE><<<dim3(tiles, L.nl), MM_R * MM_C, 0, st>>>(L, look, max_n, B, V, Tm, S, P);
       ZCSD_LAUNCH();
@@ -1024,8 +1043,8 @@ void leaf_solve(Ctx& cx, Arena& ar, const LeafTable& L, const T* B, double* lam,
       ZCSD_LAUNCH();
     }
   }
-  // a captured call looks 2 (REF_STEPS + 1) times: the state of its last look
-  // is the leaf's
+  // a captured call looks PASSES_FIXED (REF_STEPS + 1) times: the state of its
+  // last look is the leaf's
   if (sync_free) {
     leaf_last_kernel<<<ceil_div(L.nl, 256), 256, 0, st>>>(L);
     ZCSD_LAUNCH();
