@@ -11,8 +11,8 @@
 //    the bucket (the sync-free form: no host read between its launches);
 //  * H_i = sym(W_i^* A_i) and B = H_2 - H_1 per instance (the padded part of
 //    B is exactly zero), and every B of every bucket is one leaf of the
-//    batched leaf eigensolver (leaf.cu) at its own size, with a fixed number
-//    of launches and device-side convergence flags;
+//    batched leaf eigensolver (leaf.cu) at its own size, with device-side
+//    convergence flags;
 //  * C, S = diag(V^* H_i V), theta = atan2(S, C), U_i = W_i V by batched
 //    products on the padded V, then one CTA per instance sorts its angles
 //    and writes its columns into the packed outputs.
@@ -238,6 +238,7 @@ struct csd_batch {
   cudaEvent_t ev = nullptr;
   int lanes = 1;
   cudaStream_t side[MAX_LANES] = {};    // lanes 1 .. lanes - 1
+  cudaStream_t body = nullptr;          // captures the bodies of conditional nodes
   cudaEvent_t side_ev[MAX_LANES] = {};
   size_t lane_off[MAX_LANES + 1] = {};  // workspace parts, from persist_bytes
 };
@@ -415,6 +416,20 @@ void capture_all(csd_batch* b, const double* A1, const double* A2, double* U1, d
   std::memcpy(b->bound, bound, sizeof(bound));
 }
 
+// After a failure inside a capture: leaves the streams uncaptured.
+void end_captures(csd_batch* b) {
+  cudaStreamCaptureStatus cs;
+  cudaGraph_t g = nullptr;
+  // a body's graph belongs to the conditional node of the outer one
+  if (cudaStreamIsCapturing(b->body, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone)
+    cudaStreamEndCapture(b->body, &g);
+  g = nullptr;
+  if (cudaStreamIsCapturing(b->stream, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone) {
+    cudaStreamEndCapture(b->stream, &g);
+    if (g) cudaGraphDestroy(g);
+  }
+}
+
 // Per bucket engine choice (each bucket alone), then the granularity whose
 // whole batch is fastest, buckets side by side as in a later run (the sum over
 // the buckets alone counts the small ones that others hide: 48 instances of
@@ -534,7 +549,8 @@ int csd_batch_run(csd_batch* b, const double* A1, const double* A2, double* U1, 
   // already queued on the context's stream and before whatever follows it
   if (!b->stream) {
     bool ok = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming) == cudaSuccess;
+              cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming) == cudaSuccess &&
+              cudaStreamCreateWithFlags(&b->body, cudaStreamNonBlocking) == cudaSuccess;
     for (int l = 1; l < MAX_LANES; ++l)
       ok = ok && cudaStreamCreateWithFlags(&b->side[l], cudaStreamNonBlocking) == cudaSuccess &&
            cudaEventCreateWithFlags(&b->side_ev[l], cudaEventDisableTiming) == cudaSuccess;
@@ -548,6 +564,7 @@ int csd_batch_run(csd_batch* b, const double* A1, const double* A2, double* U1, 
     return CSD_ERR_CUDA;
   }
   StreamSwap swap(cx, b->stream);
+  cx.body_stream = b->body;
   for (int attempt = 0;; ++attempt) {
    try {
     if (!b->tuned) {
@@ -571,12 +588,7 @@ int csd_batch_run(csd_batch* b, const double* A1, const double* A2, double* U1, 
     return CSD_OK;
    } catch (ArenaOverflow& o) {
     // a run needed more workspace than estimated: grow it and redo the set-up
-    cudaStreamCaptureStatus cs;
-    if (cudaStreamIsCapturing(cx.stream, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone) {
-      cudaGraph_t g = nullptr;
-      cudaStreamEndCapture(cx.stream, &g);
-      if (g) cudaGraphDestroy(g);
-    }
+    end_captures(b);
     cudaStreamSynchronize(cx.stream);
     for (int l = 1; l < MAX_LANES; ++l) cudaStreamSynchronize(b->side[l]);
     cudaGetLastError();
@@ -594,12 +606,7 @@ int csd_batch_run(csd_batch* b, const double* A1, const double* A2, double* U1, 
     continue;
    } catch (CudaFail& f) {
     fprintf(stderr, "zolo_csd: CUDA error %s at %s:%d\n", cudaGetErrorString(f.err), f.file, f.line);
-    cudaStreamCaptureStatus cs;
-    if (cudaStreamIsCapturing(cx.stream, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone) {
-      cudaGraph_t g = nullptr;
-      cudaStreamEndCapture(cx.stream, &g);
-      if (g) cudaGraphDestroy(g);
-    }
+    end_captures(b);
     cudaGetLastError();
     return CSD_ERR_CUDA;
    }
@@ -618,6 +625,7 @@ int csd_batch_destroy(csd_batch* b) {
     if (b->side_ev[l]) cudaEventDestroy(b->side_ev[l]);
   }
   free_plan_ws(b);
+  if (b->body) cudaStreamDestroy(b->body);
   if (b->ev) cudaEventDestroy(b->ev);
   if (b->stream) cudaStreamDestroy(b->stream);
   delete b;

@@ -55,8 +55,7 @@ constexpr int PRE_PARTS = 32, POW_STEPS = 7;
 constexpr int J32_SMEM = 200 * 1024;    // columns of a block pair
 constexpr int REF_STEPS = 7;            // refinement steps of a pass at most, ...
 constexpr int ORTHO_STEPS = 2;          // ... the last of them only re-orthogonalise
-constexpr int PASSES = 8;               // passes of stages 1 and 2 (later ones on clusters), ...
-constexpr int PASSES_FIXED = 2;         // ... of a call without reads, where each is launched in any case
+constexpr int PASSES = 8;               // passes of stages 1 and 2 at most (later ones on clusters)
 constexpr double GAP = 4.0;             // pairs closer than this many couplings are not rotated but clustered
 constexpr int OFF_N = PASSES * (REF_STEPS + 1);  // looks at a leaf's state
 constexpr unsigned LEAF_OPEN = 1, LEAF_SKEW = 2;  // off-diagonal above rounding; X not orthonormal
@@ -640,7 +639,8 @@ __global__ void leaf_correction_kernel(LeafDev L, int it, int ortho_only, const 
       // e_ij + conj(e_ji) = -p_ij: both entries of a pair take the same branch
       const T num = sub(S[o + e], scal(lam[j], p)), mirror = sub(S[o + e], scal(lam[i], p));
       const double den = lam[j] - lam[i];
-      if (!ortho_only && fmax(abs2(num), abs2(mirror)) > tol * tol && fabs(den) > GAP * fmax(rho[i], rho[j])) v = scal(1.0 / den, num);
+      const bool apart = fabs(den) > GAP * fmax(rho[i], rho[j]);
+      if (!ortho_only && apart && fmax(abs2(num), abs2(mirror)) > tol * tol) v = scal(1.0 / den, num);
       else v = scal(-0.5, p);
     }
     E[o + e] = v;
@@ -829,10 +829,44 @@ __global__ void __cluster_dims__(JAC_CTAS, 1, 1) __launch_bounds__(JAC_THREADS)
   if (rank == 0 && tid == 0) L.done[l] = conv ? 1 : 0;
 }
 
-// the last look of a call with PASSES_FIXED passes becomes the last of all
-__global__ void leaf_last_kernel(LeafDev L) {
-  const int l = blockIdx.x * blockDim.x + threadIdx.x;
-  if (l < L.nl) L.off[l * OFF_N + OFF_N - 1] = L.off[l * OFF_N + PASSES_FIXED * (REF_STEPS + 1) - 1];
+// handle = 1 when a leaf is open at look `it` (one CTA)
+__global__ void __launch_bounds__(256) leaf_any_open_kernel(LeafDev L, int it, cudaGraphConditionalHandle handle) {
+  unsigned any = 0;
+  for (int l = threadIdx.x; l < L.nl; l += blockDim.x) any |= L.off[l * OFF_N + it];
+  any = __syncthreads_or(any != 0);
+  if (threadIdx.x == 0) cudaGraphSetConditional(handle, any ? 1u : 0u);
+}
+
+// While cx.stream is captured: what body(s) launches on the stream s becomes
+// the body of a conditional node, run when a leaf is open at look `it`.  A pass
+// of 144 launches (256 rows) that nothing needs then costs one kernel; launched
+// and left at once, as the second pass was, it took 0.2 ms.
+template <class F>
+void capture_if_open(Ctx& cx, const LeafDev& L, int it, F body) {
+  cudaStreamCaptureStatus cs;
+  cudaGraph_t graph = nullptr;
+  const cudaGraphNode_t* deps = nullptr;
+  const cudaGraphEdgeData* edges = nullptr;
+  size_t ndeps = 0;
+  ZCSD_CUDA(cudaStreamGetCaptureInfo(cx.stream, &cs, nullptr, &graph, nullptr, nullptr, nullptr));
+  cudaGraphConditionalHandle handle;
+  ZCSD_CUDA(cudaGraphConditionalHandleCreate(&handle, graph, 0, cudaGraphCondAssignDefault));
+  leaf_any_open_kernel<<<1, 256, 0, cx.stream>>>(L, it, handle);
+  ZCSD_LAUNCH();
+  ZCSD_CUDA(cudaStreamGetCaptureInfo(cx.stream, &cs, nullptr, &graph, &deps, &edges, &ndeps));
+  cudaGraphNodeParams p = {};
+  p.type = cudaGraphNodeTypeConditional;
+  p.conditional.handle = handle;
+  p.conditional.type = cudaGraphCondTypeIf;
+  p.conditional.size = 1;
+  cudaGraphNode_t node;
+  ZCSD_CUDA(cudaGraphAddNode(&node, graph, deps, edges, ndeps, &p));
+  ZCSD_CUDA(cudaStreamUpdateCaptureDependencies(cx.stream, &node, nullptr, 1, cudaStreamSetCaptureDependencies));
+  cudaGraph_t inner = p.conditional.phGraph_out[0];
+  ZCSD_CUDA(cudaStreamBeginCaptureToGraph(cx.body_stream, inner, nullptr, nullptr, 0,
+                                          cudaStreamCaptureModeThreadLocal));
+  body(cx.body_stream);
+  ZCSD_CUDA(cudaStreamEndCapture(cx.body_stream, &inner));
 }
 
 // lambda[loff_l + j] = s_jj (blockIdx.y = leaf)
@@ -844,15 +878,18 @@ __global__ void leaf_values_kernel(LeafDev L, const T* G, double* lam) {
 }
 
 template <bool CX, int NV>
-void j32_launch(cudaStream_t st, const LeafTable& L, int pass, int sweep, int round, int ctas) {
+void j32_launch(cudaStream_t st, const LeafTable& L, int pass, int sweep, int round, int ctas, bool chained) {
   constexpr int THREADS = j32_threads(128 * NV);
   static const bool attr = [] {
     ZCSD_CUDA(cudaFuncSetAttribute(j32_kernel<CX, NV, THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, J32_SMEM));
     return true;
   }();
   (void)attr;
-  launch_chained(j32_kernel<CX, NV, THREADS>, dim3(ctas, L.nl), THREADS, (size_t)L.maxcols * 128 * NV * 4, st, (const LeafDev&)L,
-                 pass, sweep, round);
+  const size_t smem = (size_t)L.maxcols * 128 * NV * 4;
+  const dim3 grid(ctas, L.nl);
+  if (chained)
+    launch_chained(j32_kernel<CX, NV, THREADS>, grid, THREADS, smem, st, (const LeafDev&)L, pass, sweep, round);
+  else j32_kernel<CX, NV, THREADS><<<grid, THREADS, smem, st>>>(L, pass, sweep, round);
   ZCSD_LAUNCH();
 }
 
@@ -954,7 +991,8 @@ void leaf_solve(Ctx& cx, Arena& ar, const LeafTable& L, const T* B, double* lam,
   const dim3 cols(ceil_div(L.maxsz, 8), L.nl);
   // Leaves of LEAF_TC rows and more take their products from gemm() when the
   // tensor cores are on (there a product costs launches and slicing, here
-  // n^3 on the FP64 pipe).  A captured call keeps to one launch for all leaves.
+  // n^3 on the FP64 pipe).  A call that may be captured keeps to one launch for
+  // all leaves.
   std::vector<int> big;
   if (!sync_free && t_tc.enabled)
     for (int l = 0; l < L.nl; ++l)
@@ -979,59 +1017,60 @@ void leaf_solve(Ctx& cx, Arena& ar, const LeafTable& L, const T* B, double* lam,
       else gemm1<T>(st, opA, OP_N, n, n, n, one, A + o, n, Bm + o, n, beta, C + o, n, 0, 0, GS_EIG);
     }
   };
-  bool any = true;
-  const int passes = sync_free ? PASSES_FIXED : PASSES;
-  for (int pass = 0; pass < passes && any; ++pass) {
+  // one pass on the stream s; false once every leaf has ended, where the host
+  // may read that
+  auto run_pass = [&](int pass, cudaStream_t s, bool reads) -> bool {
+    bool any = true;
     // two steps more of the kind at the end: stage 3 starts from S only where X is orthonormal
-    const int ortho = pass + 1 < passes ? ORTHO_STEPS : 2 * ORTHO_STEPS;
+    const int ortho = pass + 1 < PASSES ? ORTHO_STEPS : 2 * ORTHO_STEPS;
     const int look0 = pass * (REF_STEPS + 1);
     if (pass > 0) {
-      leaf_cluster_kernel<<<L.nl, 1024, 0, st>>>(L, pass);
+      leaf_cluster_kernel<<<L.nl, 1024, 0, s>>>(L, pass);
       ZCSD_LAUNCH();
-      leaf_cluster_fill_kernel<T><<<dim3(ew, L.nl), 256, 0, st>>>(L, pass, S, lds);
+      leaf_cluster_fill_kernel<T><<<dim3(ew, L.nl), 256, 0, s>>>(L, pass, S, lds);
       ZCSD_LAUNCH();
     }
     const bool one_cta = L.maxblk == 2;
     for (int sweep = 0; sweep < (one_cta ? 1 : J32_SWEEPS); ++sweep) {
       for (int r = 0; r < L.maxblk - 1; ++r) {
         switch (L.nv) {
-#define ZCSD_J32(NV) case NV: j32_launch<CX, NV>(st, L, pass, sweep, r, L.maxblk / 2); break;
+#define ZCSD_J32(NV) case NV: j32_launch<CX, NV>(s, L, pass, sweep, r, L.maxblk / 2, s == st); break;
           ZCSD_J32(1) ZCSD_J32(2) ZCSD_J32(3) ZCSD_J32(4) ZCSD_J32(5) ZCSD_J32(6) ZCSD_J32(7) ZCSD_J32(8)
           default:
             if constexpr (CX) {
-              if (L.nv == 12) j32_launch<CX, 12>(st, L, pass, sweep, r, L.maxblk / 2);
-              else j32_launch<CX, 16>(st, L, pass, sweep, r, L.maxblk / 2);
+              if (L.nv == 12) j32_launch<CX, 12>(s, L, pass, sweep, r, L.maxblk / 2, s == st);
+              else j32_launch<CX, 16>(s, L, pass, sweep, r, L.maxblk / 2, s == st);
             }
 #undef ZCSD_J32
         }
       }
     }
-    leaf_basis_kernel<T><<<cols, 256, 0, st>>>(L, pass, pass == 0 ? V : Tm, lds);
+    leaf_basis_kernel<T><<<cols, 256, 0, s>>>(L, pass, pass == 0 ? V : Tm, lds);
     ZCSD_LAUNCH();
     if (pass > 0) {  // X <- X Y
-      leaf_mm_kernel<T, MM_XY><<<dim3(tiles, L.nl), MM_R * MM_C, 0, st>>>(L, look0, max_n, B, V, Tm, S, P);
+      leaf_mm_kernel<T, MM_XY><<<dim3(tiles, L.nl), MM_R * MM_C, 0, s>>>(L, look0, max_n, B, V, Tm, S, P);
       ZCSD_LAUNCH();
       mul_big(look0 - 1, OP_N, V, Tm, P, false, zer);
-      leaf_copy_kernel<T><<<dim3(ew, L.nl), 256, 0, st>>>(L, look0 - 1, P, V);
+      leaf_copy_kernel<T><<<dim3(ew, L.nl), 256, 0, s>>>(L, look0 - 1, P, V);
       ZCSD_LAUNCH();
     }
     for (int it = 0; it <= REF_STEPS; ++it) {
       const int look = look0 + it;
-      leaf_mm_kernel<T, MM_BX><<<dim3(tiles, L.nl), MM_R * MM_C, 0, st>>>(L, look, max_n, B, V, Tm, S, P);
+      leaf_mm_kernel<T, MM_BX><<<dim3(tiles, L.nl), MM_R * MM_C, 0, s>>>(L, look, max_n, B, V, Tm, S, P);
       ZCSD_LAUNCH();
       mul_big(look - 1, OP_N, B, V, Tm, true, zer);
-      leaf_mm_kernel<T, MM_GRAM><<<dim3(tiles, L.nl, 2), MM_R * MM_C, 0, st>>>(L, look, max_n, B, V, Tm, S, P);
+      leaf_mm_kernel<T, MM_GRAM><<<dim3(tiles, L.nl, 2), MM_R * MM_C, 0, s>>>(L, look, max_n, B, V, Tm, S, P);
       ZCSD_LAUNCH();
       mul_big(look - 1, OP_C, V, Tm, S, false, zer);
       mul_big(look - 1, OP_C, V, V, P, false, zer);
-      leaf_state_kernel<T><<<cols, 256, 0, st>>>(L, look, S, P);
+      leaf_state_kernel<T><<<cols, 256, 0, s>>>(L, look, S, P);
       ZCSD_LAUNCH();
       // stop once every leaf has ended (rarely before the third look)
-      if (!sync_free && (it >= 2 || !big.empty()) && !(any = read_state(look))) break;
+      if (reads && (it >= 2 || !big.empty()) && !(any = read_state(look))) break;
       if (it == REF_STEPS) break;
-      leaf_correction_kernel<T><<<dim3(ew, L.nl), 256, 0, st>>>(L, look, it >= REF_STEPS - ortho, S, P, Tm);
+      leaf_correction_kernel<T><<<dim3(ew, L.nl), 256, 0, s>>>(L, look, it >= REF_STEPS - ortho, S, P, Tm);
       ZCSD_LAUNCH();
-      leaf_mm_kernel<T, MM_XE><<<dim3(tiles, L.nl), MM_R * MM_C, 0, st>>>(L, look, max_n, B, V, Tm, S, P);
+      leaf_mm_kernel<T, MM_XE><<<dim3(tiles, L.nl), MM_R * MM_C, 0, s>>>(L, look, max_n, B, V, Tm, S, P);
       ZCSD_LAUNCH();
       if (!big.empty()) {
         for (int l : big)
@@ -1039,15 +1078,20 @@ void leaf_solve(Ctx& cx, Arena& ar, const LeafTable& L, const T* B, double* lam,
             axpby<T>(st, L.hsz[l], L.hsz[l], 1.0, V + L.hgoff[l], L.hsz[l], 0, 0.0, P + L.hgoff[l], L.hsz[l], 0, 1);
         mul_big(look, OP_N, V, Tm, P, false, one);
       }
-      leaf_copy_kernel<T><<<dim3(ew, L.nl), 256, 0, st>>>(L, look, P, V);
+      leaf_copy_kernel<T><<<dim3(ew, L.nl), 256, 0, s>>>(L, look, P, V);
       ZCSD_LAUNCH();
     }
-  }
-  // a captured call looks PASSES_FIXED (REF_STEPS + 1) times: the state of its
-  // last look is the leaf's
-  if (sync_free) {
-    leaf_last_kernel<<<ceil_div(L.nl, 256), 256, 0, st>>>(L);
-    ZCSD_LAUNCH();
+    return any;
+  };
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (sync_free) ZCSD_CUDA(cudaStreamIsCapturing(st, &cs));
+  if (cs == cudaStreamCaptureStatusNone) {
+    for (int pass = 0; pass < PASSES && run_pass(pass, st, true); ++pass) {
+    }
+  } else {
+    run_pass(0, st, false);
+    for (int pass = 1; pass < PASSES; ++pass)
+      capture_if_open(cx, L, pass * (REF_STEPS + 1) - 1, [&](cudaStream_t s) { run_pass(pass, s, false); });
   }
   leaf_jacobi_kernel<T><<<L.nl * JAC_CTAS, JAC_THREADS, 0, st>>>(L, B, S, V, reinterpret_cast<JRec*>(L.recs),
                                                                  std::min(max_sweeps, (int)JAC_SWEEPS_MAX));

@@ -24,6 +24,7 @@ struct Plan {
 };
 
 struct Ctx {
+  cudaStream_t body_stream = nullptr;  // captures the bodies of conditional nodes (batch plans set it)
   int device = 0;
   cudaStream_t stream = nullptr;
   char* ws = nullptr;
@@ -162,8 +163,9 @@ LeafTable leaf_table_build(Ctx& cx, Arena& ar, const std::vector<long long>& bof
                            const std::vector<int>& loff, const std::vector<int>& sz, bool cplx);
 // bytes leaf_table_build takes from its arena, at most
 size_t leaf_table_bytes(const std::vector<int>& sz, bool cplx);
-// Eigenvalues to lam, eigenvectors to V (packed at goff).  sync_free: no
-// device-to-host read, for graph capture.
+// Eigenvalues to lam, eigenvectors to V (packed at goff).  sync_free: the call
+// may be captured into a graph (no device-to-host read then; passes that only
+// hard leaves need become conditional nodes, captured through cx.body_stream).
 template <class T>
 void leaf_solve(Ctx& cx, Arena& ar, const LeafTable& L, const T* B, double* lam, T* V, int max_sweeps,
                 bool sync_free);
