@@ -254,6 +254,13 @@ static void zolo_first(cudaStream_t st, Arena& ar, const Plan& pl, int n, int P,
 // An iteration in the form of Section 5, the term X (X^* X + c_j I)^{-1} = Q1
 // Q2^* / sqrt(c_j) by Householder QR of the stacked [X; sqrt(c_j) I] (2n x n,
 // row j of the lower block enters with column j): finite for every finite X.
+// It takes 20 n^3 multiply-adds a block where zolo_first takes 29.5 (r = 8;
+// the corrections to rounding are 12 of them), so on the FP64 pipe, which both
+// keep busy at large n, it is the faster first iteration from 850 rows on:
+// polar of n = 800, 900, 1400, 3000 43.8, 60.3, 173, 1418 ms against 43.1, 63.6,
+// 204, 1830; complex n = 680, 1000, 1400 107, 273, 648 against 101, 310, 762.
+// Below, its chain of n / 32 panels dominates (n = 200 12.8 ms against 2.6), and
+// on the tensor cores the chain's products are cheap at every size.
 template <class T>
 static void zolo_householder(cudaStream_t st, Arena& ar, const Plan& pl, int s, int n, int P, const T* X, T* Xn) {
   const int r = pl.r[s], m2 = 2 * n;
@@ -350,7 +357,7 @@ void zolo_pd(Ctx& cx, Arena& ar, int n, int P, const T* X0, T* W, PolarDiag* pd,
     // X is well conditioned after the first iteration; with reduced_slices its
     // Gram product and the products with the inverses then keep fewer bits of
     // their operands, the Cholesky factorizations themselves do not.
-    if (householder) {
+    if (householder || (s == 0 && !t_tc.enabled && n >= HOUSEHOLDER_MIN)) {
       zolo_householder<T>(st, ar, pl, s, n, P, X, Xn);
     } else if (s == 0) {
       zolo_first<T>(st, ar, pl, n, P, X, Xn);
@@ -832,7 +839,10 @@ size_t polar_bytes(long long n, int P, size_t es, bool tc) {
   const long long nn = n * n, r = R_MAX;
   // zolo_first's E, G, F, D per term, Z and N of two; the iterates (zolo_next
   // needs less: Z, N per term and the recursion's W, V, n^2 / 4 each at the top)
-  const long long words = nn * P * (5 * r + 8);
+  long long words = nn * P * (5 * r + 8);
+  // zolo_householder's M, E and reflectors per term, the update's partial products
+  if (!tc && n >= HOUSEHOLDER_MIN)
+    words = std::max(words, P * (2 * nn + r * (4 * nn + (n + 2 * NB_OUT) * (n + 2 * NB_OUT) + 6 * NB_OUT * n)));
   // residues of the r-term sum on the tensor cores (complex: two real terms)
   const size_t slices = tc ? tc_gemm_bytes(n, n, n, es == 8 ? (int)r : 2) * P : 0;
   return (size_t)(words * es) + slices + 64 * 256;

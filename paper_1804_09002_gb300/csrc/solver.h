@@ -12,6 +12,7 @@ namespace zcsd {
 constexpr double U_ROUND = 0x1p-53;
 constexpr double EPS_ZOLO = 1e-15;  // interval [eps, 1] of the modified Zolo-pd (Section 5.1)
 constexpr int R_MAX = 8;            // p <= 8 (Section 5)
+constexpr int HOUSEHOLDER_MIN = 850;  // rows from which Zolo-pd starts by Householder QR on the FP64 pipe (solver.cu)
 
 // Zolo-pd iteration plan (coefficients of every iteration) and the per-call
 // context: device, stream, workspace, pinned host scalars, profiler.
@@ -91,7 +92,8 @@ struct ReducedScope {
 // inverses of the Cholesky-form iterations with 45 or 51 bits of the operands
 // (tensor-core path).  householder: every iteration by Householder QR of the
 // stacked [X; sqrt(c) I], for an X0 whose Cholesky factors fail (||X0||_2 far
-// above 1; NaN in W then).  No device-to-host read, so the call can be captured
+// above 1; NaN in W then); the first iteration takes that form by itself where
+// it is the faster one.  No device-to-host read, so the call can be captured
 // in a CUDA graph.
 template <class T>
 void zolo_pd(Ctx& cx, Arena& ar, int n, int P, const T* X0, T* W, PolarDiag* pd, int stop_after = 0,
