@@ -537,7 +537,7 @@ def main():
         fp64 = {"value": v64, "unit": "s/CSD", "tflops": fl / v64 / 1e12, "steps": k64,
                 "accuracy": accuracy(R64, A1, A2, th_known, n, dev), "clocks": ck64}
         ctx.set_tensor_cores(bool(args.tc))
-    # ---- mixed precision (fewer slices in the well-conditioned Cholesky
+    # ---- mixed precision (fewer operand bits in the well-conditioned Cholesky
     # iteration), same workload and accuracy checks
     mixed = None
     if args.tc and args.mixed_slices in (5, 6) and not cfg["cplx"]:

@@ -195,7 +195,7 @@ int zolo_plan(double ell0, int rmax, int max_iter, int* r_out, double* ell_out);
 
 /* Kernel accounting, for roofline reports (not needed for computing).
  * Kinds: 0 = GEMM (FP64 FMA tiles), 1 = Householder QR panel, 2 = Cholesky
- * diagonal block, 3 = Jacobi leaves, 4 = tensor-core FP64 GEMM (sliced BF16
+ * diagonal block, 3 = Jacobi leaves, 4 = tensor-core FP64 GEMM (modular BF16
  * products on tcgen05; `flops` counts the FP64-equivalent 2mnk).  While enabled, each launch of these
  * kernels is bracketed by CUDA events on the context stream; `flops` sums
  * the multiply-add work each launch executes (2 per real FMA, 8 per complex
@@ -206,13 +206,16 @@ typedef struct {
   long long count[5];
   double ms[5];
   double flops[5];
-  /* GEMM launches split by call site (0 other, 1-3 QR panel update, 4-6 Q
-   * formation, 7 Zolotarev term sum, 8 Gram matrix, 9-10 Cholesky, 11-14
-   * triangular solves, 15 H, 16 orthogonality check, 17 Zolo-eig,
-   * 18 assembly, 19 Algorithm 2, 20 merging of the blocked QR's WY factors,
-   * 21 rows of the dense block X in the trailing update of the stacked
-   * [X; sqrt(c) I] QR factorization; site 3 holds the rows below it;
-   * 22 csd_polar_backward) */
+  /* GEMM launches split by call site: 0 other, 1-3 QR panel update, 4-6 Q
+   * formation, 7 Zolotarev term sum, 8 Gram matrix, 9 inverse Cholesky
+   * factor, 10 its trailing update, 11 sum of the inverses in a
+   * Cholesky-form iteration, 12 bases of the first iteration, 13 product of X
+   * with the sum, 14 Gram matrix of the lower halves of the bases, 15 H,
+   * 16 orthogonality check, 17 Zolo-eig, 18 assembly, 19 Algorithm 2,
+   * 20 merging of the blocked QR's WY factors, 21 corrections of the bases to
+   * orthonormality, 22 csd_polar_backward.  The numbers 9 to 14 and 21 once
+   * named products of replaced algorithms (Cholesky rows and triangular
+   * solves; the upper rows of the stacked QR, now in 3). */
   long long site_count[24];
   double site_ms[24];
   double site_flops[24];
@@ -341,7 +344,7 @@ int csd_set_test_hooks(csd_ctx* ctx, unsigned flags, long long tc_probe_wait, in
 
 /* C = alpha op(A) op(B) + beta C in real FP64 on this library's product
  * kernels: engine 0 = the FP64-pipe tiles, engine 1 = the tensor-core kernel
- * (exact BF16 slicing, FP64-accurate; any m, n, k).  The building block of
+ * (exact modular BF16 products, FP64-accurate; any m, n, k).  The building block of
  * every step of Zolo-pd and Zolo-eig; it is not itself a step of the paper.
  *   opA, opB: 0 = N, 1 = T.  A (lda >= rows of A), B (ldb), C (ldc >= m)
  *   are column-major DEVICE pointers (a host pointer returns -8/-10/-13).

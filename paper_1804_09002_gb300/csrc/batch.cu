@@ -249,7 +249,7 @@ size_t bucket_bytes(const Bucket& bk) {
   const long long P = (long long)bk.inst.size(), nb = bk.nb, nn = nb * nb;
   const size_t es = sizeof(double);
   size_t b = (size_t)(2 * P * nn * 3 + P * nn * 4 + P * nb * 4) * es + (size_t)bk.leaves.vtot * 4 * es;
-  // zolo_pd on 2P problems plus the tensor-core slices of its largest product
+  // zolo_pd on 2P problems plus the tensor-core residues of its largest product
   b += (size_t)(nn * 2 * P * (6 * R_MAX + 6)) * es;
   if (nb >= HOUSEHOLDER_MIN) b += (size_t)(nn * 2 * P * R_MAX) * es;  // the Householder form of the first iteration
   b += tc_gemm_bytes(nb, nb, nb, R_MAX) * 2 * P;

@@ -112,8 +112,8 @@ void count_launch();
 // (chain_wait), and a CTA that has only its results left to write lets the
 // successor's CTAs in (chain_next; a CTA that exits counts too).  A kernel
 // launched without the attribute waits as ever, and so does whatever follows a
-// chained kernel without it.  csd n = 64 1.50 -> 1.38 ms, n = 500 14.2 -> 12.6,
-// n = 1024 39.0 -> 35.6, polar n = 2048 40.7 -> 37.8.
+// chained kernel without it.  csd n = 64 1.50 -> 1.37 ms, n = 500 14.5 -> 12.9,
+// n = 1024 38.9 -> 35.5, polar n = 2048 41.2 -> 38.3.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

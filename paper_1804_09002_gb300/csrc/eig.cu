@@ -370,8 +370,12 @@ void heig_impl(Ctx& cx, Arena& ar, int n, const T* Bin, int ldb, double* lam, T*
       // contiguous runs, each padded to its largest size nb.  A group's time
       // is modelled as a latency term growing with nb (the sequential panel
       // and Cholesky steps) plus work per padded problem, t = a nb + c Pa
-      // nb^3 (a = 0.065 ms, c = 9e-9 ms for real data, fitted to measured
-      // group times on GB300); the cuts minimise the modelled total.
+      // nb^3; the cuts minimise the modelled total and depend on c / a only.
+      // a = 0.065 ms and c = 9e-9 ms (real data) describe an earlier build on
+      // the tensor cores; groups of 1100 and 3000 rows now take 19 and 90 ms
+      // there (a = 0.016, c = 1.6e-9: the ratio within a third), but 132 and
+      // 2090 ms on the FP64 pipe (a = 0.03, c = 7e-8), where the cuts pad more
+      // than they should.
       std::sort(act.begin(), act.end(), [&](int a, int b) {
         return work[a].b.sz != work[b].b.sz ? work[a].b.sz > work[b].b.sz : work[a].b.off < work[b].b.off;
       });
@@ -630,7 +634,7 @@ void heig_impl(Ctx& cx, Arena& ar, int n, const T* Bin, int ldb, double* lam, T*
     }
     ar.release(mlev);
   }
-  // ---- leaves: batched two-sided Jacobi on every block <= eig_leaf; scalar
+  // ---- leaves: the batched leaf eigensolver on every block <= eig_leaf; scalar
   // blocks keep their diagonal
   std::vector<int> jo, js;
   for (size_t i = 0; i < leaf_off.size(); ++i) {

@@ -29,8 +29,8 @@
 // B itself; stage 1 only supplies the starting basis.
 //
 // Measured on GB300 against cyclic FP64 Jacobi with two launches per round
-// (heig of a random matrix): n = 64 6.3 -> 0.9 ms, 200 31 -> 2.6 ms; complex
-// n = 512 14.6 ms.  At n = 1024 one leaf takes 21 ms (54 ms without tensor
+// (heig of a random matrix): n = 64 6.3 -> 0.8 ms, 200 31 -> 2.1 ms; complex
+// n = 512 9.4 ms.  At n = 1024 one leaf takes 16 ms (41 ms without tensor
 // cores) where splitting down to 256 rows took 125 ms, hence the leaf size.
 // Stage 1 is then 70 % of the time, bound by the issue slots of the few SMs
 // that hold a leaf; the refinement's products run at 60 % of the FP64 pipe.
@@ -990,7 +990,7 @@ void leaf_solve(Ctx& cx, Arena& ar, const LeafTable& L, const T* B, double* lam,
   const int ew = std::max(1, std::min(ceil_div((long long)L.maxsz * L.maxsz, 256), 304));
   const dim3 cols(ceil_div(L.maxsz, 8), L.nl);
   // Leaves of LEAF_TC rows and more take their products from gemm() when the
-  // tensor cores are on (there a product costs launches and slicing, here
+  // tensor cores are on (there a product costs launches and conversions, here
   // n^3 on the FP64 pipe).  A call that may be captured keeps to one launch for
   // all leaves.
   std::vector<int> big;

@@ -8,7 +8,8 @@
 namespace zcsd {
 
 // Split-K factor for a product whose output alone gives too few tiles, or a
-// tile count that fills its last wave poorly: the GEMM keeps two CTAs per SM
+// tile count that fills its last wave poorly, for tiles of 4096 outputs (gemm()
+// may take smaller ones, which need less of a split): the GEMM keeps two CTAs per SM
 // resident (304 slots on 152 SMs), so a launch of C CTAs runs ceil(C / 304)
 // waves; pick the split s (K chunks of at least kmin) that maximises the
 // filled fraction C s / (304 ceil(C s / 304)), smaller s on ties.

@@ -17,8 +17,8 @@ namespace zcsd {
 
 // Workspace of one Zolo-pd call (P = 1) for n <= CSD_NOALLOC_MAX_N, complex
 // FP64 (the larger element type), plus the input/output staging of polar():
-// about 4 MiB at n = 64 (panels of at most 96 rows take no split-K
-// partial products); 6 MiB leaves headroom.
+// the bases, Gram matrices and corrections of eight terms (polar_bytes), about
+// 4 MiB at n = 64; 6 MiB leaves headroom.
 constexpr size_t NOALLOC_BYTES = (size_t)6 << 20;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_BYTES];
@@ -60,7 +60,7 @@ thread_local int t_hi[4096];
 // The call runs polar_impl (the polar() entry point's body) on an arena over
 // the static scratch.  The thread's tensor-core dispatch state and profiler
 // are switched off for the call and restored afterwards, so a product can
-// never draw slices from another call's arena (n <= 64 is also below the
+// never draw operands from another call's arena (n <= 64 is also below the
 // tensor-core kernel's smallest tile).
 template <class T>
 int polar_noalloc_impl(int n, const T* A, int lda, T* Wo, int ldw, T* Ho, int ldh, cudaStream_t st, void* base) {

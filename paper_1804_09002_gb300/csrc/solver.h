@@ -47,7 +47,7 @@ struct Ctx {
   int sign_mode = 0;            // 1: canonical column signs of U1, U2, V1 (csd_set_sign_convention)
   double alg2_svd_factor = 1e3;  // SVD polar fallback when ||R~ - R|| / ||R|| > factor n u (< 0: never)
   int eig_leaf = LEAF;           // Zolo-eig blocks of at most this size go to the Jacobi leaf solver
-  int mixed_slices = 7;          // BF16 slices of the Cholesky-iteration products (5, 6 or 7)
+  int mixed_slices = 7;          // Cholesky-iteration products keep 45 (5), 51 (6) or 56 (7) operand bits
   unsigned mixed_scope = 0;      // bit 0: the CSD's / polar()'s Zolo-pd, bit 1: Zolo-eig's Zolo-pd
 };
 
