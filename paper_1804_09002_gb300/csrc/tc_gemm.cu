@@ -745,11 +745,15 @@ struct CombArgs {
 
 // C = alpha 2^(ea + eb - 2 bits) x + beta Cin, x = P frac(sum_t R_t / p_t) with
 // the fraction in [-1/2, 1/2): the sum of R_t round(2^96 / p_t) mod 2^96, good
-// to 2^-85 of P.  A block covers 128 rows x 16 columns, four rows per thread.
+// to 2^-85 of P.  A block covers 128 rows x 16 columns, four rows per thread;
+// WIDE numbers the column blocks in the grid's first dimension, where there are
+// too many for the second (with one numbering for both, a division in each
+// block, the kernel lost a fifth of its rate).
 // Reads and writes 2 nmod + 8 bytes per entry; bound by the integer pipe
 // (three 32 x 32 + 64-bit multiply-adds per modulus).
+template <bool WIDE>
 __global__ void __launch_bounds__(256) tc_combine_kernel(const CombArgs g, const __grid_constant__ RnsTab tab) {
-  const int m0 = blockIdx.x * TC_BM, c0 = blockIdx.y * 16, z = blockIdx.z;
+  const int m0 = (WIDE ? blockIdx.y : blockIdx.x) * TC_BM, c0 = (WIDE ? blockIdx.x : blockIdx.y) * 16, z = blockIdx.z;
   if (g.uplo == 1 && m0 > c0 / TC_BN * TC_BN + TC_BN - 1) return;
   const bool failed = *g.err != 0;
   const int row = m0 + 4 * (threadIdx.x & 31);
@@ -951,7 +955,9 @@ void tc_gemm(const GemmArgs<double>& g, cudaStream_t st, Arena& ar, int* err) {
   c.alpha = re(g.alpha); c.beta = re(g.beta);
   c.Cin = g.Cin; c.ldcin = g.ldcin; c.bdivC = g.bdivC; c.sCin = g.sCin;
   c.C = g.C; c.ldc = g.ldc; c.sC = g.sC; c.es = g.es; c.err = err;
-  tc_combine_kernel<<<dim3(t.tiles_m, ceil_div(g.n, 16), g.batch), 256, 0, st>>>(c, tab);
+  const int cblk = ceil_div(g.n, 16);
+  if (cblk <= 65535) tc_combine_kernel<false><<<dim3(t.tiles_m, cblk, g.batch), 256, 0, st>>>(c, tab);
+  else tc_combine_kernel<true><<<dim3(cblk, t.tiles_m, g.batch), 256, 0, st>>>(c, tab);
   ZCSD_LAUNCH();
   if (tok.slot >= 0) {
     // FP64-equivalent multiply-add work over the tiles executed

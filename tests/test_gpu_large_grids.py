@@ -1,5 +1,6 @@
 """Products with so many columns that their tiles do not fit a grid's second
-dimension (65535): 8-column tiles of the FP64 pipe from 524 281 columns on."""
+dimension (65535): 8-column tiles of the FP64 pipe from 524 281 columns on,
+16-column blocks of the tensor-core product's combination from 1 048 561 on."""
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -17,7 +18,7 @@ def ctx():
     c.close()
 
 
-@pytest.mark.parametrize("engine,m,n", [(0, 1, 524281), (0, 3, 700001), (0, 33, 600001)])
+@pytest.mark.parametrize("engine,m,n", [(0, 1, 524281), (0, 3, 700001), (0, 33, 600001), (1, 3, 1048577)])
 def test_very_wide_product(ctx, engine, m, n):
     """Small integers, so that every engine is exact."""
     k = 2
