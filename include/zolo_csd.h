@@ -336,8 +336,9 @@ int csd_set_zolo_control(csd_ctx* ctx, int max_extra_passes, int stop_after);
  *     copy or MMA; the wait runs out, the launch writes NaN outputs, sets
  *     the device error flag and the call returns CSD_ERR_DEVICE_TIMEOUT.
  *     The context stays usable.
- *   tc_flush_every: accepted and without effect (the partial sums of long
- *     products need no write-out).
+ *   tc_flush_every > 0: the tensor-core kernel reduces its running residue
+ *     sums every this many drains of 256 k (default: every 32768 drains, i.e.
+ *     only for k above 8 million, where the sums would outgrow FP32).
  * Returns 0, -1 (NULL context), -2 (unknown flag), -3 / -4 (negative). */
 #define CSD_TEST_REJECT_EIG_SPLITS 1u
 int csd_set_test_hooks(csd_ctx* ctx, unsigned flags, long long tc_probe_wait, int tc_flush_every);

@@ -913,6 +913,7 @@ int run_with_ws(Ctx& cx, size_t need, csd_info* info, F body) {
       t_tc.ar = &ar;
       t_tc.err = tc_err;
       t_tc.probe_wait = cx.tc_probe_wait;
+      t_tc.flush_every = cx.tc_flush_every;
       status = body(ar);
       if (tc_err) {
         int h = 0;

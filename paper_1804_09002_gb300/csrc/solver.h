@@ -42,7 +42,7 @@ struct Ctx {
   int zolo_stop_after = 0;    // polar(): > 0 returns the iterate X_k after k iterations (k <= plan steps)
   unsigned test_flags = 0;    // TEST_* below (fault injection on the host; default off)
   long long tc_probe_wait = 0;  // tensor-core kernel: polls of a barrier nothing signals (0 = none)
-  int tc_flush_every = 0;       // accepted and without effect (csd_set_test_hooks)
+  int tc_flush_every = 0;       // tensor-core kernel: drains between reductions of the running sum (0 = default)
   bool force_tc_err = false;    // the running call needs the tensor-core error flag (csd_gemm)
   int sign_mode = 0;            // 1: canonical column signs of U1, U2, V1 (csd_set_sign_convention)
   double alg2_svd_factor = 1e3;  // SVD polar fallback when ||R~ - R|| / ||R|| > factor n u (< 0: never)

@@ -50,6 +50,7 @@ constexpr int TC_A_STAGE = TC_BM * TC_BK * 2;
 constexpr int TC_STAGE = TC_A_STAGE + TC_BN * TC_BK * 2;
 constexpr int TC_SMEM = TC_NSTAGE * TC_STAGE + 1024;
 constexpr int TC_DRAIN = 256 / TC_BK;  // stages between reductions of an accumulator
+constexpr int TC_FOLD = 32768;  // drains between reductions of their sum: 257 x 32769 < 2^24 stays exact in FP32
 constexpr int TC_EPI_WARPS = 16;
 constexpr int TC_THREADS = 32 * (2 + TC_EPI_WARPS);
 constexpr int TC_CPT = TC_BN / 4;  // accumulator columns per epilogue thread
@@ -277,6 +278,7 @@ struct TcArgs {
   int nrbA, nrbB, nkb;       // 128-row blocks of the operands, 64-k blocks
   int batch, bstrideA, bstrideB;  // problems; 0: all problems share that operand
   int kb_flags, uplo, nmod;
+  int fold;                  // drains between reductions of the running sum (TC_FOLD at most)
   int tiles_m, tiles_n, tiles;  // output tiles, and those that uplo keeps (per problem and modulus)
   const __nv_bfloat16 *A, *B;
   unsigned short* R;         // [problem][modulus][n][128 tiles_m] residues
@@ -320,6 +322,9 @@ __device__ __forceinline__ TcItem tc_item(const TcArgs& g, long long it) {
   return t;
 }
 
+// FOLD: some item has more drains than g.fold, so its running sum is reduced on
+// the way (the others' code is without it).
+template <bool FOLD>
 __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcArgs g, const __grid_constant__ RnsTab tab) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -469,6 +474,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcArgs g, 
       f32x2 acc[TC_CPT / 2];
 #pragma unroll
       for (int c = 0; c < TC_CPT / 2; ++c) acc[c] = 0ull;
+      int left = g.fold;
       for (int q = 0; q < Q; q += TC_DRAIN, ++cycle) {
         // uniform over the warp: the TMEM accesses below are warp-collective
         ok = __all_sync(0xffffffffu, !*abort_v && mbar_wait(smem_u32(&accf_bar[cycle & 1u]), (cycle >> 1) & 1u, abort_v));
@@ -496,6 +502,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcArgs g, 
             acc[(16 * h + c) / 2] = add2(
                 acc[(16 * h + c) / 2],
                 mod_p2(pack2(__uint_as_float(r[h & 1][c]), __uint_as_float(r[h & 1][c + 1])), np2, inv2, mg2, nmg2));
+        }
+        if (FOLD && --left == 0) {
+          left = g.fold;
+#pragma unroll
+          for (int c = 0; c < TC_CPT / 2; ++c) acc[c] = mod_p2(acc[c], np2, inv2, mg2, nmg2);
         }
       }
       if (!ok) break;
@@ -896,6 +907,7 @@ void tc_gemm(const GemmArgs<double>& g, cudaStream_t st, Arena& ar, int* err) {
   unsigned short* R = ar.get<unsigned short>((size_t)g.batch * tab.nmod * g.n * ldr);
   t.A = A; t.B = B; t.R = R; t.err = err;
   t.probe_wait = t_tc.probe_wait;
+  t.fold = t_tc.flush_every > 0 ? std::min(t_tc.flush_every, TC_FOLD) : TC_FOLD;
   // inner-dimension balance (one term only): e_k bounds row k of op(B);
   // op(A) D and D^-1 op(B) with D = diag(2^e_k) have the same product, and
   // per-row / per-column scaling of the balanced operands is accurate
@@ -942,11 +954,15 @@ void tc_gemm(const GemmArgs<double>& g, cudaStream_t st, Arena& ar, int* err) {
     convert(b, b, 1, nB);
   }
   static std::once_flag attr_once;
-  std::call_once(attr_once,
-                 [] { cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM); });
+  std::call_once(attr_once, [] {
+    cudaFuncSetAttribute(tc_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
+    cudaFuncSetAttribute(tc_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
+  });
   const long long items = (long long)t.tiles * tab.nmod * g.batch;
   const int grid = (int)std::min<long long>(items, num_sms());
-  tc_gemm_kernel<<<grid, TC_THREADS, TC_SMEM, st>>>(t, tab);
+  const bool fold = (long long)t.nkb * nsum > (long long)t.fold * TC_DRAIN;
+  if (!fold) tc_gemm_kernel<false><<<grid, TC_THREADS, TC_SMEM, st>>>(t, tab);
+  else tc_gemm_kernel<true><<<grid, TC_THREADS, TC_SMEM, st>>>(t, tab);
   ZCSD_LAUNCH();
   CombArgs c{};
   c.m = g.m; c.n = g.n; c.ldr = ldr; c.uplo = t.uplo; c.tiles_m = t.tiles_m;

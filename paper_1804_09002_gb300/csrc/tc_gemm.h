@@ -14,6 +14,7 @@ struct TcState {
   Arena* ar = nullptr;
   int* err = nullptr;
   long long probe_wait = 0;  // > 0: each launch first polls a barrier nothing signals (timeout-path tests)
+  int flush_every = 0;       // > 0: drains between reductions of the running residue sums (tests of that path)
   unsigned reduced_sites = 0;  // bit s: call site s keeps reduced_bits bits of an operand instead of 56
   int reduced_bits = 56;
 };
