@@ -326,16 +326,23 @@ RNS_PRODUCTS = 14
 
 # DRAM traffic of the tensor-core product kernel per launch, from one ncu
 # capture (dram__bytes_read.sum + dram__bytes_write.sum over every launch of
-# the kernel in one step), with the hash of the kernel source it was taken
-# at; reported only while tc_gemm.cu is unchanged since the capture.
-TRAFFIC = {"tc_gemm": {"bytes_per_launch": 396064809, "src_hash": "b20b1f9c2d56235e",
+# the kernel in one step), with the hash of the sources it was taken at, the
+# kernel's and those that choose its launches; reported only while they are
+# unchanged since the capture.
+TRAFFIC = {"tc_gemm": {"bytes_per_launch": 396064809, "src_hash": "70e7a7fad080a612",
                       "profile": "profiles/tc_gemm_kernel_csd_n4096_traffic.md"}}
+
+
+LAUNCH_SOURCES = ["solver.cu", "eig.cu", "leaf.cu", "linalg.cu", "blas.cu", "tc_gemm.h", "linalg.h", "solver.h"]
 
 
 def _src_hash(name):
     import hashlib
-    with open(os.path.join(ROOT, "paper_1804_09002_gb300", "csrc", name), "rb") as f:
-        return hashlib.sha256(f.read()).hexdigest()[:16]
+    h = hashlib.sha256()
+    for s in [name] + LAUNCH_SOURCES:
+        with open(os.path.join(ROOT, "paper_1804_09002_gb300", "csrc", s), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
 
 
 def traffic_for(kernel):
