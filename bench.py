@@ -329,7 +329,7 @@ RNS_PRODUCTS = 14
 # the kernel in one step), with the hash of the sources it was taken at, the
 # kernel's and those that choose its launches; reported only while they are
 # unchanged since the capture.
-TRAFFIC = {"tc_gemm": {"bytes_per_launch": 396064809, "src_hash": "70e7a7fad080a612",
+TRAFFIC = {"tc_gemm": {"bytes_per_launch": 396340648, "src_hash": "20a09da8c503a8c4",
                       "profile": "profiles/tc_gemm_kernel_csd_n4096_traffic.md"}}
 
 
@@ -556,7 +556,7 @@ def main():
         mixed = {"value": vx, "unit": "s/CSD", "tflops": fl / vx / 1e12, "steps": kmx,
                  "slices": args.mixed_slices, "scope": args.mixed_scope,
                  "accuracy": accuracy(Rx, A1, A2, th_known, n, dev), "clocks": ckx,
-                 "what": "Gram and triangular-solve products of the Cholesky-form Zolo-pd iteration with "
+                 "what": "Gram product and products with the inverses of the Cholesky-form Zolo-pd iteration with "
                          f"{45 if args.mixed_slices == 5 else 51} bits; everything else FP64-accurate (56)"}
         ctx.set_mixed_precision(7, 0)
     # ---- e2e: same call with pinned host buffers (copies inside the call)

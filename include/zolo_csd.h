@@ -38,7 +38,8 @@ extern "C" {
 
 #define CSD_OK 0
 #define CSD_ERR_CUDA 1            /* a CUDA call failed (context may be lost) */
-#define CSD_ERR_NOT_CONVERGED 2   /* polar(): the Zolo-pd iterate did not converge (last iterate written) */
+#define CSD_ERR_NOT_CONVERGED 2   /* polar(): the Zolo-pd iterate did not converge (last iterate written);
+                                   * csd_polar: a polar factor stayed non-finite and the SVD fallback is off */
 #define CSD_WARN_ALG2_RCHECK 3    /* Algorithm 2: ||R~ - R|| above tolerance (Section 5.1) */
 #define CSD_ERR_EIG_SPLIT 4       /* Zolo-eig could not split a block after retries */
 #define CSD_ERR_NONFINITE 5       /* input holds NaN or Inf */
@@ -272,7 +273,8 @@ int csd_set_mixed_precision(csd_ctx* ctx, int slices, unsigned scope);
  * backward stable, and info->alg2_used[i] = 2.  Default factor 1e3; 0 makes
  * every block that takes Algorithm 2 use the SVD; a negative factor
  * disables the fallback, and a block above 1e3 n u then returns
- * CSD_WARN_ALG2_RCHECK as a warning.  The SVD costs O(n^3) per sweep and
+ * CSD_WARN_ALG2_RCHECK as a warning (CSD_ERR_NOT_CONVERGED where the quotient
+ * is not finite).  The SVD costs O(n^3) per sweep and
  * some ten sweeps.  Returns 0, -1 (NULL context) or -2 (NaN). */
 int csd_set_alg2_fallback(csd_ctx* ctx, double factor);
 

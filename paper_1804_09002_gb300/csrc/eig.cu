@@ -209,10 +209,12 @@ std::vector<X> download(Ctx& cx, const X* d, size_t count) {
   return h;
 }
 
-// ||X_p - shift_p I||_F^2 of every problem of a reduction table (device out)
+// ||X_p - shift_p I||_F^2 of every problem of a reduction table (device out),
+// each by `parts` CTAs
 template <class T>
 void blk_fro2(cudaStream_t st, Arena& ar, const T* X, int ld, const std::vector<long long>& boff,
-              const std::vector<int>& m, const std::vector<int>& c, const double* dshift, double* out) {
+              const std::vector<int>& m, const std::vector<int>& c, const double* dshift, double* out,
+              int parts = RED_PARTS) {
   const int P = (int)boff.size();
   if (P == 0) return;
   RedTab t;
@@ -220,10 +222,10 @@ void blk_fro2(cudaStream_t st, Arena& ar, const T* X, int ld, const std::vector<
   t.m = upload(ar, st, m);
   t.c = upload(ar, st, c);
   t.shift = dshift;
-  double* part = ar.get<double>((size_t)P * RED_PARTS);
-  blk_fro2_partial<T><<<dim3(RED_PARTS, P), 256, 0, st>>>(X, ld, t, part);
+  double* part = ar.get<double>((size_t)P * parts);
+  blk_fro2_partial<T><<<dim3(parts, P), 256, 0, st>>>(X, ld, t, part);
   ZCSD_LAUNCH();
-  blk_finish<<<P, 256, 0, st>>>(part, RED_PARTS, out);
+  blk_finish<<<P, 256, 0, st>>>(part, parts, out);
   ZCSD_LAUNCH();
 }
 
@@ -566,7 +568,10 @@ void heig_impl(Ctx& cx, Arena& ar, int n, const T* Bin, int ldb, double* lam, T*
           double* doffa = ar.get<double>(2 * cand.size());
           blk_fro2<T>(st, ar, Om, nb, boff, rm, rc, nullptr, doffa);
           const std::vector<int> whole(cand.size(), nb);
-          if (!householder) blk_fro2<T>(st, ar, Nf, nb, eoff, whole, whole, nullptr, doffa + cand.size());  // E1
+          // E1, by 64 entries a thread on up to two CTAs per SM (32 CTAs: 0.3 ms at 1500 rows)
+          if (!householder)
+            blk_fro2<T>(st, ar, Nf, nb, eoff, whole, whole, nullptr, doffa + cand.size(),
+                        (int)std::min<long long>(304, std::max<long long>(RED_PARTS, nbb / 16384)));
           const std::vector<double> h = download(cx, doffa, (householder ? 1 : 2) * cand.size());
           std::vector<int> accept(Pa, 0), retry;
           bool any_acc = false, redo = false;
